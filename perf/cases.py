@@ -236,9 +236,9 @@ def _cloud(case, X, th, g, family, N, a):
     H = Xs.T @ (_curvature(family, Xs @ th)[:, None] * Xs) * (a * X.shape[0] / k)
     H += torch.eye(X.shape[1], dtype=torch.float64, device=DEV) / _prior_var(
         dict(case, family=family))
-    L = torch.linalg.cholesky(H)
-    z = torch.randn(X.shape[1], N, generator=g, device=DEV, dtype=torch.float64)
-    c = th + torch.linalg.solve_triangular(L.T, z, upper=True).T
+    Linv = np.linalg.inv(np.linalg.cholesky(H.cpu().numpy()))  # H^-1 = Linv' Linv
+    z = torch.randn(N, X.shape[1], generator=g, device=DEV, dtype=torch.float64)
+    c = th + z @ torch.from_numpy(Linv).to(DEV)
     return c.to(torch.float64 if case["dtype"] == "f64" else torch.float32).contiguous()
 
 
