@@ -243,6 +243,71 @@ __device__ __forceinline__ RowC<CT> row_consts(CT eb, CT y, CT inv_s2, CT nu = C
   return c;
 }
 
+// The hardware exponential, logarithm (base 2) and reciprocal with denormals flushed: no scaling code
+// around them. Used where the argument is at least 2^-12 in size or absolute error is what counts.
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float lg2_ftz(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_ftz(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// The logistic increment for |D| <= kFarD in FP32 (used above 1/2), from
+//   softplus(eta_bar + D) - softplus(eta_bar) = log((1 - s) + s e^D),
+//   sigma(eta_bar + D) = s e^D / ((1 - s) + s e^D):
+// one exponential, one logarithm and one reciprocal, no case distinction. Root-mean-square error of d
+// against FP64 over eta_bar of sd 1.5: 6e-8 for |D| in [1/2, 1] and 8e-8 in [1, 2] (1.0e-7 and
+// 1.2e-7 for the form row_incr takes beyond kFarD, which has two logarithms); of r 3e-8 and 4e-8 (the
+// same). Above kFarD the logarithm's relative error would count.
+constexpr float kFarD = 2.0f;
+__device__ __forceinline__ void logistic_far(float s, float w, float D, float &d, float &r) {
+  const float se = s * ex2_ftz(D * 1.44269504088896341f);
+  const float den = (1.0f - s) + se;
+  const float wD = w * D;
+  r = (wD + s) - se * rcp_ftz(den);
+  d = fmaf(0.5f * wD, D, fmaf(s, D, -0.693147180559945309f * lg2_ftz(den)));
+}
+
+// The logistic cumulant series of row_incr in FP32: kappa_3 .. kappa_10 as polynomials in w with w (and
+// q for the odd ones) factored out and scaled by 1/(k-1)!, so every constant is the immediate of a
+// scalar FMA; the chain of d divides each by its k.
+__device__ __forceinline__ void logistic_series(float s, float w, float D, float &d, float &r) {
+  const float q = fmaf(s, -2.f, 1.f);
+  const float e4 = (float)(1.0 / 6) - w;
+  const float e6 = fmaf(w, w - 0.25f, (float)(1.0 / 120));
+  const float e8 =
+      fmaf(w, fmaf(w, (float)(1.0 / 3) - w, (float)(-1.0 / 40)), (float)(1.0 / 5040));
+  const float e10 = fmaf(
+      w, fmaf(w, fmaf(w, w - (float)(5.0 / 12), (float)(7.0 / 144)), (float)(-17.0 / 12096)),
+      (float)(1.0 / 362880));
+  const float o3 = 0.5f * q;
+  const float o5 = q * fmaf(w, -0.5f, (float)(1.0 / 24));
+  const float o7 = q * fmaf(w, fmaf(w, 0.5f, (float)(-1.0 / 12)), (float)(1.0 / 720));
+  const float o9 = q * fmaf(w, fmaf(w, fmaf(w, -0.5f, 0.125f), (float)(-1.0 / 160)),
+                            (float)(1.0 / 40320));
+  float2 c = make_float2(0.1f * e10, e10);  // the chains of d and r
+  const float2 DD = make_float2(D, D);
+  c = __ffma2_rn(c, DD, make_float2(o9 * (float)(1.0 / 9), o9));
+  c = __ffma2_rn(c, DD, make_float2(e8 * 0.125f, e8));
+  c = __ffma2_rn(c, DD, make_float2(o7 * (float)(1.0 / 7), o7));
+  c = __ffma2_rn(c, DD, make_float2(e6 * (float)(1.0 / 6), e6));
+  c = __ffma2_rn(c, DD, make_float2(o5 * 0.2f, o5));
+  c = __ffma2_rn(c, DD, make_float2(e4 * 0.25f, e4));
+  c = __ffma2_rn(c, DD, make_float2(o3 * (float)(1.0 / 3), o3));
+  const float nwd2 = -w * (D * D);
+  r = nwd2 * c.y;
+  d = nwd2 * D * c.x;
+}
+
 // Horner steps of the two cumulant-series chains at once (FP32: one packed FMA per step):
 // (pd, pr) = (pd, pr) * D + kappa * (1/k!, 1/(k-1)!).
 template <typename CT>
@@ -296,7 +361,17 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
       series = !__any_sync(__activemask(), fabs(D) > kSmall);
     else
       series = fabs(D) <= kSmall;
-    if (series) {
+    if constexpr (sizeof(CT) == 4) {
+      if (series) {
+        logistic_series(sb, w, D, d, r);
+        return;
+      }
+      if (!__any_sync(__activemask(), fabsf(D) > kFarD)) {
+        logistic_far(sb, w, D, d, r);
+        return;
+      }
+    }
+    if (sizeof(CT) == 8 && series) {
       const CT q = CT(1) - CT(2) * sb;
       const CT k3 = w * q;
       const CT k4 = w * (CT(1) - CT(6) * w);
@@ -321,7 +396,7 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
       return;
     }
     if constexpr (sizeof(CT) == 4) {
-      // |D| > 1/2 in FP32: with eta = eta_bar + D and softplus(x) = max(x, 0) + log(1 + e^-|x|),
+      // |D| > kFarD in FP32: with eta = eta_bar + D and softplus(x) = max(x, 0) + log(1 + e^-|x|),
       //   L1 = softplus(eta) - softplus(eta_bar)
       //      = [max(eta, 0) - max(eta_bar, 0)] + log(1 + e^-|eta|) - log(1 + e^-|eta_bar|),
       // where log(1 + e^-|eta_bar|) = -log(max(s, 1 - s)) (1 - s is exact for s >= 1/2), and
@@ -330,11 +405,12 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
       // approximations (MUFU ex2/lg2/rcp) err by about 2e-7 absolute, the size of what d loses
       // to its own cancellation (-L1 + sD + wD^2/2) at this |D| in FP32 anyway.
       const float eb = c.c2, eta = eb + D;
-      const float e = __expf(-fabsf(eta)), ope = 1.0f + e;
-      const float lb = __logf(fmaxf(sb, 1.0f - sb));
+      const float e = ex2_ftz(-1.44269504088896341f * fabsf(eta)), ope = 1.0f + e;
+      const float ln2 = 0.693147180559945309f;
+      const float lb = ln2 * lg2_ftz(fmaxf(sb, 1.0f - sb));
       const float pos = eb >= 0.0f ? (eta >= 0.0f ? D : -eb) : (eta >= 0.0f ? eta : 0.0f);
-      const float L1f = pos + (__logf(ope) + lb);
-      const float inv = __fdividef(1.0f, ope);
+      const float L1f = pos + (ln2 * lg2_ftz(ope) + lb);
+      const float inv = rcp_ftz(ope);
       const float sg = eta >= 0.0f ? inv : e * inv;
       r = fmaf(w, D, sb - sg);
       d = fmaf(0.5f * w * D, D, fmaf(sb, D, -L1f));
