@@ -1870,8 +1870,9 @@ int smc_batch_init(smc_batch **out, int32_t P, const smc_problem *probs, const s
   // default warps per CTA for its p and m (res_default_warps; more when none fits), unless its
   // configuration asks for the streamed trajectory (hmc_kernel = 1)
   {
-    static const int kCand4[][2] = {{0, 8},  {7, 12},  {1, 16},  {6, 20},
-                                    {2, 24}, {3, 32},  {9, 40}};
+    // {tile, covariate slots} by warps per CTA
+    static const int kCand4[][2] = {{0, 8},  {7, 12}, {1, 16},  {6, 20}, {2, 24},
+                                    {3, 32}, {9, 40}, {24, 56}, {25, 64}};
     static const int kCand2[][2] = {{10, 8}, {11, 12}, {12, 16}, {13, 20},
                                     {14, 24}, {15, 32}, {16, 40}};
     static const int kCand1[][2] = {{17, 8}, {18, 12}, {19, 16}, {20, 20},
@@ -1884,7 +1885,8 @@ int smc_batch_init(smc_batch **out, int32_t P, const smc_problem *probs, const s
       const smc_ctx *c = b->ctx[q];
       for (int w = res_default_warps(c->p, c->m); w <= 4 && gt[q] < 0; w *= 2) {
         const int(*cand)[2] = w == 1 ? kCand1 : w == 2 ? kCand2 : kCand4;
-        for (int t = 0; t < 7; ++t)
+        const int ncand = w == 4 ? 9 : 7;
+        for (int t = 0; t < ncand; ++t)
           if (c->p <= cand[t][1] && res_launch_batch_bf16(cand[t][0], dry, c->p, c->m, c->G,
                                                           b->stream, c->sms, true) == 0) {
             gt[q] = cand[t][0];

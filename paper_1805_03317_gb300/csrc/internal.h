@@ -130,8 +130,10 @@ constexpr int kTwoWarpRows = 512;
 // Warps per CTA of the default resident tile for p covariates and m subsample rows (measured on
 // GB300, 1024 particles per problem): one warp while a warp's rows outweigh the per-pass work
 // that every warp repeats (p 9..24 up to m = 400, p > 24 up to m = 160; at p <= 8 two warps
-// always do better), two up to m = 512, else four.
+// always do better), two up to m = 512, else four. Above 40 covariates four (us per trajectory of
+// L = 20 at p = 50: 229 against 241 with eight at m = 1250, 100 against 176 at m = 512).
 inline int res_default_warps(int p, int m) {
+  if (p > 40) return 4;
   if (p > 8 && m <= (p <= 24 ? 400 : 160)) return 1;
   return m <= kTwoWarpRows ? 2 : 4;
 }
@@ -142,6 +144,10 @@ int res_launch_batch_bf16_w2(int tile, const BatchArgs &b, int p_max, int m_max,
 int res_launch_bf16_w1(int tile, const EstArgs &a, cudaStream_t s, int sms, bool dry);
 int res_launch_batch_bf16_w1(int tile, const BatchArgs &b, int p_max, int m_max, int G_max,
                              cudaStream_t s, int sms, bool dry);
+// The wide tiles (24, 25: 41 to 64 covariates) of the BF16 table.
+int res_launch_bf16_wide(int tile, const EstArgs &a, cudaStream_t s, int sms, bool dry);
+int res_launch_batch_bf16_wide(int tile, const BatchArgs &b, int p_max, int m_max, int G_max,
+                               cudaStream_t s, int sms, bool dry);
 
 // Stage kernels (stage.cu). All return cudaError_t.
 int pack_rows(const void *X, int x_dtype, int64_t n, int p, int64_t ld, const void *y, void *Xp,
