@@ -328,15 +328,14 @@ int moments_at(smc_ctx *c, const double *theta_d, double *A_out, double *B_out, 
 }
 
 __global__ void k_log_post(int p, const double *theta, const double *mu, const double *var,
-                           const double *A, double *out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double lp = *A;
-    for (int c = 0; c < p; ++c) {
-      const double r = theta[c] - mu[c];
-      lp += -0.5 * r * r / var[c];
-    }
-    *out = lp;
+                           const double *A, double *out) {  // one warp
+  double lp = 0.0;
+  for (int c = threadIdx.x; c < p; c += 32) {
+    const double r = theta[c] - mu[c];
+    lp += -0.5 * r * r / var[c];
   }
+  for (int o = 16; o; o >>= 1) lp += __shfl_xor_sync(0xffffffffu, lp, o);
+  if (threadIdx.x == 0) *out = *A + lp;
 }
 
 __global__ void k_scale(int count, double f, double *v) {
@@ -392,7 +391,12 @@ int newton_iterate(smc_ctx *c, double *theta_d, int64_t stride, double tol) {
                                c->stream));
     CUDA_OK(c, cudaStreamSynchronize(c->stream));
     if (info) return fail(c, SMC_ERR_NONFINITE, "Newton step: negative Hessian not positive definite");
-    double t = 1.0;
+    double t = 1.0, smax = 0.0;
+    for (int k = 0; k < p; ++k) smax = fmax(smax, fabs(sh[k]));
+    if (smax < tol) {  // the last step: too short for the objective to tell its ends apart
+      LAUNCH(c, axpy_vec(p, theta_d, 1.0, step, theta_d, c->stream), 1);
+      break;
+    }
     while (true) {
       LAUNCH(c, axpy_vec(p, theta_d, t, step, cand, c->stream), 1);
       if ((r = moments_strided(c, cand, A1, stride))) return r;

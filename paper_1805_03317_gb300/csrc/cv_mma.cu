@@ -147,9 +147,12 @@ __global__ void __launch_bounds__(kRows) k_cv_mma(const __nv_bfloat16 *Xp, int64
   double *lps = ths + 128;
   double *Cacc = lps + kRows;
   double *red = Cacc + ((np + 1) & ~1);
-  uint64_t *bar = reinterpret_cast<uint64_t *>(red + 32);
+  double *lgt = red + 32;
+  uint64_t *bar = reinterpret_cast<uint64_t *>(lgt + (FAM == 2 ? kLgTable : 0));
   uint32_t *tptr = reinterpret_cast<uint32_t *>(bar + 1);
 
+  const double lc = row_value_const<FAM>(s2, nu);
+  if (FAM == 2) lgamma_table(lgt);
   for (int c = tid; c < 128; c += kRows) ths[c] = c < p ? theta[c] : 0.0;
   for (int q = tid; q < np; q += kRows) Cacc[q] = 0.0;
   // strips that no copy or write ever fills stay zero
@@ -204,7 +207,7 @@ __global__ void __launch_bounds__(kRows) k_cv_mma(const __nv_bfloat16 *Xp, int64
         }
         const double eta = ((ep[0] + ep[1]) + (ep[2] + ep[3])) + ((ep[4] + ep[5]) + (ep[6] + ep[7]));
         const RowC<float> *tl = reinterpret_cast<const RowC<float> *>(Xp + (r0 + k) * S + Yo);
-        row_value<FAM>(eta, (double)__ldg(&tl->y), s2, nu, l, d1, d2);
+        row_value<FAM>(eta, (double)__ldg(&tl->y), s2, nu, lc, lgt, l, d1, d2);
       }
       Aacc += l;
       lps[k] = d1;
@@ -327,29 +330,34 @@ int tmem_cols(int N) {
   return c;
 }
 
-size_t cv_mma_smem(int p, int N) {
+size_t cv_mma_smem(int p, int N, int fam) {
   const int np = p * (p + 1) / 2;
   return (size_t)kM / 8 * kStrip + (size_t)3 * (N / 8) * kStrip +
-         sizeof(double) * (128 + kRows + ((np + 1) & ~1) + 32) + 16;
+         sizeof(double) * (128 + kRows + ((np + 1) & ~1) + 32 + (fam == 2 ? kLgTable : 0)) + 16;
 }
 
 template <int FAM>
 int launch_fam(const __nv_bfloat16 *Xp, int64_t n, int p, int S, int Yo, double s2, double nu,
                const double *theta, double *part, int maxblocks, int *nblocks, cudaStream_t s) {
   const int N = ((p + 15) / 16) * 16;
-  const size_t smem = cv_mma_smem(p, N);
+  const size_t smem = cv_mma_smem(p, N, FAM);
   cudaError_t e = cudaFuncSetAttribute(k_cv_mma<FAM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return (int)e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cv_mma<FAM>, kRows, smem);
+  e = cudaFuncSetAttribute(k_cv_mma<FAM>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return (int)e;
-  if (per_sm < 1) return (int)cudaErrorInvalidConfiguration;
-  int dev = 0, sms = 0;
+  int dev = 0, sms = 0, sm_smem = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  // CTAs per SM by shared memory (1 KB of it per CTA is the system's) and tensor memory. The occupancy
+  // query answers 1 for kernels that allocate tensor memory; a tile's phases (copy, FP64 row terms,
+  // MMAs, B) follow one another in a CTA, so several CTAs per SM are what overlaps them: logistic
+  // n = 10^6, p = 20: 774 us with one, 393 us with three and one exponential per row.
+  int per_sm = sm_smem / (int)(smem + 1024);
   const int cols = tmem_cols(N);
   if (per_sm * cols > 512) per_sm = 512 / cols;  // every resident CTA gets its columns at once
+  if (per_sm < 1) per_sm = 1;
   const int64_t ntiles = (n + kRows - 1) / kRows;
   int64_t grid = (int64_t)per_sm * sms;
   if (grid > maxblocks) grid = maxblocks;

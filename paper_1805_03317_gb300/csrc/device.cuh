@@ -505,30 +505,45 @@ __device__ __forceinline__ double row_l2_any(int fam, const RowC<double> &c, dou
   }
 }
 
-// Full per-row value and derivatives at eta (used by the moment kernel, FP64). s2: the Gaussian
-// variance or the Student-t squared scale; nu: the Student-t degrees of freedom.
+// Full per-row value and derivatives at eta (used by the moment kernels, FP64). s2: the Gaussian
+// variance or the Student-t squared scale; nu: the Student-t degrees of freedom. An FP64 logarithm,
+// exponential or lgamma costs a warp one to several thousand cycles on this part, so what does not
+// depend on eta comes in ready: lc = row_value_const (once per thread) and the table of log k!
+// (lgamma_table, once per block), and the logistic value and derivatives share one exponential.
+template <int FAM> __device__ __forceinline__ double row_value_const(double s2, double nu) {
+  if (FAM == 4)
+    return lgamma(0.5 * (nu + 1.0)) - lgamma(0.5 * nu) - 0.5 * log(3.14159265358979323846 * nu * s2);
+  if (FAM == 3) return -0.5 * log(6.283185307179586476925286766559 * s2);
+  return 0.0;
+}
+// log(k!) = lgamma(k + 1), k < kLgTable, for the Poisson responses (whole block; sync after).
+constexpr int kLgTable = 64;
+__device__ __forceinline__ void lgamma_table(double *lgt) {
+  for (int k = threadIdx.x; k < kLgTable; k += blockDim.x) lgt[k] = lgamma((double)k + 1.0);
+}
 template <int FAM>
-__device__ __forceinline__ void row_value(double eta, double y, double s2, double nu, double &l,
-                                          double &d1, double &d2) {
+__device__ __forceinline__ void row_value(double eta, double y, double s2, double nu, double lc,
+                                          const double *lgt, double &l, double &d1, double &d2) {
   if (FAM == 4) {
     const double r = y - eta, q = fma(r, r, nu * s2);
-    l = lgamma(0.5 * (nu + 1.0)) - lgamma(0.5 * nu) - 0.5 * log(3.14159265358979323846 * nu * s2) -
-        0.5 * (nu + 1.0) * log1p(r * r / (nu * s2));
+    l = lc - 0.5 * (nu + 1.0) * log1p(r * r / (nu * s2));
     d1 = (nu + 1.0) * r / q;
     d2 = (nu + 1.0) * (r * r - nu * s2) / (q * q);
   } else if (FAM == 0) {
-    const double s = sigmoid_(eta);
-    l = y * eta - softplus_(eta);
+    const double e = exp(-fabs(eta)), inv = 1.0 / (1.0 + e);
+    const double s = eta >= 0.0 ? inv : e * inv;
+    l = y * eta - (fmax(eta, 0.0) + log1p(e));
     d1 = y - s;
     d2 = -s * (1.0 - s);
   } else if (FAM == 2) {
     const double mu = exp(eta);
-    l = y * eta - mu - lgamma(y + 1.0);
+    const int k = (int)fmin(fmax(y, 0.0), (double)(kLgTable - 1));
+    l = y * eta - mu - ((double)k == y ? lgt[k] : lgamma(y + 1.0));
     d1 = y - mu;
     d2 = -mu;
   } else if (FAM == 3) {
     const double r = y - eta;
-    l = -0.5 * log(6.283185307179586476925286766559 * s2) - r * r / (2.0 * s2);
+    l = lc - r * r / (2.0 * s2);
     d1 = r / s2;
     d2 = -1.0 / s2;
   } else {

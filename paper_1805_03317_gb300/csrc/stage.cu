@@ -169,12 +169,15 @@ __global__ void __launch_bounds__(kCvThreads) k_cv_partials(const XT *Xp, int64_
   double *ths = sh;                                   // [p]
   double *d1s = ths + p;                              // [kCvTile]
   double *red = d1s + kCvTile;                        // [32]
-  AT *xs = reinterpret_cast<AT *>(red + 32);          // [kCvTile][p]
+  double *lgt = red + 32;                             // [kLgTable] (Poisson)
+  AT *xs = reinterpret_cast<AT *>(lgt + kLgTable);    // [kCvTile][p]
   AT *wx = xs + kCvTile * p;                          // [kCvTile][p]   l'' * x
   AT *d2s = wx + kCvTile * p;                         // [kCvTile]
   const int tid = threadIdx.x;
   const int np = p * (p + 1) / 2;
   for (int c = tid; c < p; c += blockDim.x) ths[c] = theta[c];
+  if (fam == 2) lgamma_table(lgt);
+  const double lc = fam == 4 ? row_value_const<4>(s2, nu) : fam == 3 ? row_value_const<3>(s2, nu) : 0.0;
   int qr[MAXQ], qc[MAXQ];
   double acc[MAXQ];
 #pragma unroll
@@ -214,11 +217,11 @@ __global__ void __launch_bounds__(kCvThreads) k_cv_partials(const XT *Xp, int64_
         for (int c = 0; c < p; ++c) eta = fma((double)xs[tid * p + c], ths[c], eta);
         const double y = packed_y<XT>(Xp + k * S, Yo);
         switch (fam) {
-          case 0: row_value<0>(eta, y, s2, nu, l, d1, d2); break;
-          case 1: row_value<1>(eta, y, s2, nu, l, d1, d2); break;
-          case 2: row_value<2>(eta, y, s2, nu, l, d1, d2); break;
-          case 3: row_value<3>(eta, y, s2, nu, l, d1, d2); break;
-          default: row_value<4>(eta, y, s2, nu, l, d1, d2); break;
+          case 0: row_value<0>(eta, y, s2, nu, lc, lgt, l, d1, d2); break;
+          case 1: row_value<1>(eta, y, s2, nu, lc, lgt, l, d1, d2); break;
+          case 2: row_value<2>(eta, y, s2, nu, lc, lgt, l, d1, d2); break;
+          case 3: row_value<3>(eta, y, s2, nu, lc, lgt, l, d1, d2); break;
+          default: row_value<4>(eta, y, s2, nu, lc, lgt, l, d1, d2); break;
         }
       }
       d1s[tid] = d1;
@@ -303,10 +306,9 @@ cudaError_t launch_cv(int need, int nblocks, size_t smem, cudaStream_t s, const 
   return launch_cv_q<XT, 32>(nblocks, smem, s, Xp, n, p, S, Yo, fam, s2, nu, theta, part);
 }
 
-int cv_moments_blocks(int p) {
-  (void)p;
-  return 2 * 152;
-}
+// Partial blocks: at most two per SM, four for the tensor-core kernel on narrow rows (their partials
+// are small and four CTAs fit an SM).
+int cv_moments_blocks(int p) { return (p <= 64 ? 4 : 2) * 152; }
 
 int cv_moments(const void *Xp, int x_dtype, int64_t n, int p, int S, int Yo, int fam, double sigma2,
                double nu, const double *theta, double *partials, int nblocks, double *A, double *B,
@@ -321,8 +323,9 @@ int cv_moments(const void *Xp, int x_dtype, int64_t n, int p, int S, int Yo, int
     return (int)cudaGetLastError();
   }
   if (p * (p + 1) / 2 > kCvThreads * kCvMaxPairs) return (int)cudaErrorInvalidValue;
+  if (nblocks > 2 * 152) nblocks = 2 * 152;
   const size_t at = x_dtype == 0 ? sizeof(double) : sizeof(float);
-  const size_t smem = (size_t)(p + kCvTile + 32) * sizeof(double) + (2 * kCvTile * p + kCvTile) * at;
+  const size_t smem = (size_t)(p + kCvTile + 32 + kLgTable) * sizeof(double) + (2 * kCvTile * p + kCvTile) * at;
   const int np = p * (p + 1) / 2, need = (np + kCvThreads - 1) / kCvThreads;
   cudaError_t e;
   if (x_dtype == 0)
@@ -342,7 +345,8 @@ int cv_moments(const void *Xp, int x_dtype, int64_t n, int p, int S, int Yo, int
 
 // ------------------------------------------------------------------------------------------------
 // Dense FP64 Cholesky of a p x p SPD matrix held in shared memory by one block (right-looking).
-// Returns false (on every thread) if a pivot is not positive.
+// Returns false (on every thread) if a pivot is not positive. chol_block: one root and one division
+// per column entry, as FP64 states want it (their runs are compared to the last digits).
 // ------------------------------------------------------------------------------------------------
 __device__ bool chol_block(double *M, int p, int *flag) {
   const int tid = threadIdx.x, bs = blockDim.x;
@@ -376,48 +380,79 @@ __device__ bool chol_block(double *M, int p, int *flag) {
   return true;
 }
 
+// The same for Newton steps and FP32 states, with the reciprocal diagonal in rd [p]. A warp-wide FP64
+// instruction holds its sub-partition's pipe for 64 cycles however few lanes need it, so a column is
+// one reciprocal square root and one barrier (each warp takes the root for itself), the trailing
+// rows updated with 32 lanes across from the unscaled column, M[i, k] -= M[i, j] M[k, j] / v, and the
+// columns are scaled once, at the end. p = 20, a Newton step: 66 us with chol_block and one thread's
+// substitutions, 27 us with this and a warp's.
+__device__ bool chol_fast(double *M, int p, double *rd) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  for (int j = 0; j < p; ++j) {
+    const double v = M[j * p + j];  // final: the previous column's update ended with a barrier
+    if (!(v > 0.0) || !isfinite(v)) return false;  // uniform: every thread reads the same pivot
+    const double rv = rsqrt(v), iv = rv * rv;
+    for (int i = j + 1 + warp; i < p; i += nw) {
+      const double f = M[i * p + j] * iv;
+      for (int k = j + 1 + lane; k <= i; k += 32) M[i * p + k] -= f * M[k * p + j];
+    }
+    if (tid == 0) rd[j] = rv;
+    __syncthreads();
+  }
+  for (int i = warp; i < p; i += nw)
+    for (int k = lane; k < p; k += 32) M[i * p + k] = k > i ? 0.0 : M[i * p + k] * rd[k];
+  __syncthreads();
+  return true;
+}
+
 // Newton step for the posterior mode: solve (-C + diag(1/v)) step = B - (theta - mu)/v.
 __global__ void k_newton_step(int p, const double *theta, const double *B, const double *C,
                               const double *mu, const double *var, double *step, int *info) {
   extern __shared__ double M[];
-  __shared__ int flag;
-  double *g = M + p * p;
-  const int tid = threadIdx.x;
+  double *g = M + p * p, *rd = g + p;
+  const int tid = threadIdx.x, lane = tid & 31;
   for (int c = tid; c < p; c += blockDim.x) g[c] = B[c] - (theta[c] - mu[c]) / var[c];
   // M = -C + diag(1/var) + lam I. A log-density that is not concave (Student-t far from the mode)
   // can leave M indefinite; lam = 1e-8 max|diag| (times 10 per retry) then keeps the step an
   // ascent direction (Levenberg's damping). Uniform across the block: every thread sees the same
   // factorisation outcome.
-  double scale = 0.0;
-  for (int i = 0; i < p; ++i) scale = fmax(scale, fabs(-C[i * p + i] + 1.0 / var[i]));
-  if (!(scale > 0.0)) scale = 1e-300;
   double lam = 0.0;
   bool ok = false;
   for (int tries = 0; tries < 40 && !ok; ++tries) {
+    if (tries == 1) {
+      double scale = 0.0;
+      for (int i = 0; i < p; ++i) scale = fmax(scale, fabs(-C[i * p + i] + 1.0 / var[i]));
+      lam = 1e-8 * (scale > 0.0 ? scale : 1e-300);
+    }
+    __syncthreads();
     for (int e = tid; e < p * p; e += blockDim.x) {
       const int i = e / p, k = e % p;
       M[e] = -C[e] + (i == k ? 1.0 / var[i] + lam : 0.0);
     }
     __syncthreads();
-    ok = chol_block(M, p, &flag);
-    lam = lam == 0.0 ? 1e-8 * scale : 10.0 * lam;
+    ok = chol_fast(M, p, rd);
+    if (tries) lam = 10.0 * lam;
   }
   if (!ok) {
     if (tid == 0) *info = 1;
     return;
   }
-  if (tid == 0) {  // forward then back substitution (p <= 126: one thread is enough)
+  if (tid < 32) {  // forward then back substitution by one warp, an unknown at a time
     for (int i = 0; i < p; ++i) {
-      double s = g[i];
-      for (int k = 0; k < i; ++k) s -= M[i * p + k] * g[k];
-      g[i] = s / M[i * p + i];
+      const double x = g[i] * rd[i];
+      __syncwarp();
+      for (int k = i + 1 + lane; k < p; k += 32) g[k] -= M[k * p + i] * x;
+      if (lane == 0) g[i] = x;
+      __syncwarp();
     }
     for (int i = p - 1; i >= 0; --i) {
-      double s = g[i];
-      for (int k = i + 1; k < p; ++k) s -= M[k * p + i] * g[k];
-      g[i] = s / M[i * p + i];
+      const double x = g[i] * rd[i];
+      __syncwarp();
+      for (int k = lane; k < i; k += 32) g[k] -= M[i * p + k] * x;
+      if (lane == 0) g[i] = x;
+      __syncwarp();
     }
-    *info = 0;
+    if (lane == 0) *info = 0;
   }
   __syncthreads();
   for (int c = tid; c < p; c += blockDim.x) step[c] = g[c];
@@ -426,11 +461,11 @@ __global__ void k_newton_step(int p, const double *theta, const double *B, const
 int newton_step(int p, const double *theta, const double *B, const double *C, const double *mu,
                 const double *var, double *step, double *work, int *info, cudaStream_t s) {
   (void)work;
-  const size_t smem = (size_t)(p * p + p) * sizeof(double);
+  const size_t smem = (size_t)(p * p + 2 * p) * sizeof(double);
   cudaError_t e =
       cudaFuncSetAttribute(k_newton_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
-  k_newton_step<<<1, 256, smem, s>>>(p, theta, B, C, mu, var, step, info);
+  k_newton_step<<<1, 128, smem, s>>>(p, theta, B, C, mu, var, step, info);
   return (int)cudaGetLastError();
 }
 
@@ -1313,12 +1348,21 @@ int weighted_moments(int is_f64, int N, int p, const double *W, const void *thet
 // Mass matrix: Cholesky of Sigma with the jitter schedule 1e-10 tr/p, x10 per retry (added
 // cumulatively, at most 12 retries); then Linv = chol^{-1} for drawing rho = Linv' z. When no
 // retry succeeds (e.g. a single particle: Sigma = 0) the previous mass matrix is kept.
+// Whether the factor and its inverse both fit shared memory, and the shared bytes of k_mass.
+__host__ __device__ inline bool mass_two(int p) { return p <= 112; }
+inline size_t mass_smem(int p) {
+  return (size_t)((mass_two(p) ? 2 : 1) * p * p + p) * sizeof(double);
+}
 template <typename CT>
 __device__ __forceinline__ void k_mass_body(int p, const double *Sigma_in, double *Sigma,
     double *chol, CT *Sigma_ct, CT *Linv_ct, double *work, DevState *st, int bid_, int nblk_) {
   extern __shared__ double M[];
-  __shared__ int flag;
   __shared__ double jit;
+  constexpr bool EXACT = sizeof(CT) == 8;
+  __shared__ int flag;
+  // FP32 states: the reciprocal diagonal, then L^-1 in shared memory where both matrices fit, else
+  // in the global work matrix
+  double *rd = M + p * p, *X = mass_two(p) ? rd + p : work;
   const int tid = threadIdx.x;
   for (int e = tid; e < p * p; e += blockDim.x) work[e] = Sigma_in[e];
   if (tid == 0) {
@@ -1332,7 +1376,7 @@ __device__ __forceinline__ void k_mass_body(int p, const double *Sigma_in, doubl
   while (true) {
     for (int e = tid; e < p * p; e += blockDim.x) M[e] = work[e];
     __syncthreads();
-    ok = chol_block(M, p, &flag);
+    ok = EXACT ? chol_block(M, p, &flag) : chol_fast(M, p, rd);
     if (ok || tries == 12) break;
     ++tries;
     __syncthreads();
@@ -1349,18 +1393,35 @@ __device__ __forceinline__ void k_mass_body(int p, const double *Sigma_in, doubl
     Sigma_ct[e] = (CT)work[e];
   }
   __syncthreads();
-  // column j of Linv by forward substitution, L X = I (FP64 in work; each thread owns columns)
-  for (int j = tid; j < p; j += blockDim.x) {
-    for (int i = 0; i < j; ++i) work[i * p + j] = 0.0;
-    work[j * p + j] = 1.0 / M[j * p + j];
-    for (int i = j + 1; i < p; ++i) {
-      double acc = 0.0;
-      for (int k = j; k < i; ++k) acc += M[i * p + k] * work[k * p + j];
-      work[i * p + j] = -acc / M[i * p + i];
+  if constexpr (EXACT) {
+    // column j of Linv by forward substitution, L X = I (FP64 in work; each thread owns columns)
+    for (int j = tid; j < p; j += blockDim.x) {
+      for (int i = 0; i < j; ++i) work[i * p + j] = 0.0;
+      work[j * p + j] = 1.0 / M[j * p + j];
+      for (int i = j + 1; i < p; ++i) {
+        double acc = 0.0;
+        for (int k = j; k < i; ++k) acc += M[i * p + k] * work[k * p + j];
+        work[i * p + j] = -acc / M[i * p + i];
+      }
     }
+    __syncthreads();
+    for (int e = tid; e < p * p; e += blockDim.x) Linv_ct[e] = (CT)work[e];
+  } else {
+    // L X = I by forward substitution, one row of X per step: a warp per remaining row, lanes over
+    // the columns (p steps of one dependent FMA and a barrier instead of p^2 / 2 in one thread per
+    // column; p = 20, the whole mass matrix: 45 us before, 35 us now)
+    const int lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    for (int e = tid; e < p * p; e += blockDim.x) X[e] = e / p == e % p ? 1.0 : 0.0;
+    __syncthreads();
+    for (int i = 0; i < p; ++i) {
+      for (int r = i + 1 + warp; r < p; r += nw) {
+        const double f = M[r * p + i] * rd[i];
+        for (int c = lane; c <= i; c += 32) X[r * p + c] -= f * X[i * p + c];
+      }
+      __syncthreads();
+    }
+    for (int e = tid; e < p * p; e += blockDim.x) Linv_ct[e] = (CT)(X[e] * rd[e / p]);
   }
-  __syncthreads();
-  for (int e = tid; e < p * p; e += blockDim.x) Linv_ct[e] = (CT)work[e];
 }
 template <typename CT>
 __global__ void k_mass(int p, const double *Sigma_in, double *Sigma, double *chol, CT *Sigma_ct,
@@ -1370,7 +1431,7 @@ __global__ void k_mass(int p, const double *Sigma_in, double *Sigma, double *cho
 
 int mass_matrix(int is_f64, int p, const double *Sigma_in, double *Sigma, double *chol,
                 void *Sigma_ct, void *Linv_ct, double *work, DevState *st, cudaStream_t s) {
-  const size_t smem = (size_t)p * p * sizeof(double);
+  const size_t smem = mass_smem(p);
   cudaError_t e;
   if (is_f64) {
     e = cudaFuncSetAttribute(k_mass<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1816,7 +1877,9 @@ int stage_batch(const StageBatch &sb, cudaStream_t s, int64_t *launches) {
   kb_sum_mean<<<sb.total[kSkSumMean], 256, 0, s>>>(sb.args, off(kSkSumMean), P);
   kb_cov_partials<<<sb.total[kSkMom], kMomThreads, 0, s>>>(sb.args, off(kSkMom), P);
   kb_sum_cov<<<sb.total[kSkSumCov], 256, 0, s>>>(sb.args, off(kSkSumCov), P);
-  const size_t smem = (size_t)sb.max_p * sb.max_p * sizeof(double);
+  // (the largest of the problems' plans; past 112 covariates one matrix fits, below both)
+  size_t smem = mass_smem(sb.max_p);
+  if (!mass_two(sb.max_p) && mass_smem(112) > smem) smem = mass_smem(112);
   cudaError_t e =
       cudaFuncSetAttribute(kb_mass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
