@@ -100,6 +100,26 @@ __device__ __forceinline__ void ld16(uint32_t taddr, float *v) {
 #pragma unroll
   for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(r[e]);
 }
+// The same in two parts, so that a load is in flight while the columns before it are worked on: the
+// registers hold the values only after ld16_wait, which names them so that no use moves ahead of it.
+__device__ __forceinline__ void ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+      "%12, %13, %14, %15}, [%16];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void ld16_wait(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                 "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
+                 "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
 __device__ __forceinline__ uint32_t bf(float v) {
   return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v));
 }
@@ -117,14 +137,9 @@ __device__ __forceinline__ void fam_terms(float eta, float y, float inv_s2, floa
   if (FAM == 4) {  // Student-t: -(nu+1)/2 log(1 + r^2 / (nu s^2)), (nu+1) r / (nu s^2 + r^2)
     const float r = y - eta, z = r * r * inv_s2;
     l = -0.5f * (nu + 1.f) * log1pf(z / nu);
-    d1 = __fdividef((nu + 1.f) * r * inv_s2, nu + z);
-  } else if (FAM == 0) {  // logistic: y eta - softplus(eta), y - sigma(eta)
-    const float e = __expf(-fabsf(eta));
-    const float inv = __fdividef(1.f, 1.f + e);
-    l = y * eta - (fmaxf(eta, 0.f) + __logf(1.f + e));
-    d1 = y - (eta >= 0.f ? inv : e * inv);
+    d1 = (nu + 1.f) * r * inv_s2 * rcp_ftz(nu + z);
   } else if (FAM == 2) {  // Poisson: y eta - e^eta
-    const float mu = __expf(eta);
+    const float mu = ex2_ftz(1.44269504088896341f * eta);
     l = y * eta - mu;
     d1 = y - mu;
   } else if (FAM == 3) {  // Gaussian: -(y - eta)^2 / (2 sigma^2)
@@ -137,6 +152,52 @@ __device__ __forceinline__ void fam_terms(float eta, float y, float inv_s2, floa
     log_phi_(s * eta, lp, lam);
     l = lp;
     d1 = s * lam;
+  }
+}
+
+// l and l' of 16 columns (d) and their sum of l. ok: bit e = column e counts.
+template <int FAM>
+__device__ __forceinline__ float fam_chunk(const uint32_t (&v)[16], const float *y, float inv_s2,
+                                           float nu, uint32_t ok, float (&d)[16]) {
+  if constexpr (FAM == 0) {
+    // Logistic: l = y eta - max(eta, 0) - log(1 + e^-|eta|), l' = y - s with s = 1 / (1 + e^-eta); the
+    // last term is log max(s, 1 - s), so the 16 columns need one logarithm, of the product of those
+    // (each in [1/2, 1]): two special-function operations per column instead of three, and the
+    // rest two columns per instruction.
+    const float2 one = make_float2(1.f, 1.f), mone = make_float2(-1.f, -1.f);
+    const float2 nl2e = make_float2(-1.44269504088896341f, -1.44269504088896341f);
+    float2 P = one, ls = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int e = 0; e < 16; e += 2) {
+      const float2 et = make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+      const float2 ye = make_float2(y[e], y[e + 1]);
+      float2 s = __fmul2_rn(et, nl2e);
+      s = __fadd2_rn(make_float2(ex2_ftz(s.x), ex2_ftz(s.y)), one);
+      s = make_float2(rcp_ftz(s.x), rcp_ftz(s.y));
+      float2 dd = __ffma2_rn(s, mone, ye);
+      const float2 om = __ffma2_rn(s, mone, one);
+      float2 mm = make_float2(fmaxf(s.x, om.x), fmaxf(s.y, om.y));
+      float2 a = __ffma2_rn(ye, et, make_float2(fminf(-et.x, 0.f), fminf(-et.y, 0.f)));
+      if (ok != 0xFFFFu) {
+        if (!(ok >> e & 1u)) dd.x = a.x = 0.f, mm.x = 1.f;
+        if (!(ok >> (e + 1) & 1u)) dd.y = a.y = 0.f, mm.y = 1.f;
+      }
+      P = __fmul2_rn(P, mm);
+      ls = __fadd2_rn(ls, a);
+      d[e] = dd.x;
+      d[e + 1] = dd.y;
+    }
+    return fmaf(0.693147180559945309f, lg2_ftz(P.x * P.y), ls.x + ls.y);
+  } else {
+    float ls = 0.f;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      float l = 0.f;
+      d[e] = 0.f;
+      if (ok >> e & 1u) fam_terms<FAM>(__uint_as_float(v[e]), y[e], inv_s2, nu, l, d[e]);
+      ls += l;
+    }
+    return ls;
   }
 }
 
@@ -154,9 +215,11 @@ __device__ __forceinline__ void split8(const float *d, uint4 &hi, uint4 &lo) {
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const __nv_bfloat162 hb = __floats2bfloat162_rn(d[2 * q], d[2 * q + 1]);
-    const float2 hf = __bfloat1622float2(hb);
-    const __nv_bfloat162 lb = __floats2bfloat162_rn(d[2 * q] - hf.x, d[2 * q + 1] - hf.y);
     h[q] = *reinterpret_cast<const uint32_t *>(&hb);
+    const float2 rest = __ffma2_rn(make_float2(__uint_as_float(h[q] << 16),
+                                               __uint_as_float(h[q] & 0xFFFF0000u)),
+                                   make_float2(-1.f, -1.f), make_float2(d[2 * q], d[2 * q + 1]));
+    const __nv_bfloat162 lb = __floats2bfloat162_rn(rest.x, rest.y);
     l[q] = *reinterpret_cast<const uint32_t *>(&lb);
   }
   hi = make_uint4(h[0], h[1], h[2], h[3]);
@@ -294,23 +357,28 @@ __global__ void __launch_bounds__(kThreads) k_full_mma(
       {
         const float *yt = ys + b * kR;
         const bool fast = full_p && t0 + kR <= r1;
-        for (int c0 = half * 64; c0 < half * 64 + 64; c0 += 16) {
-          float v[16], d[16];
-          ld16(tE + tlane + (uint32_t)c0, v);
+        const int c_lo = half * 64;
+        uint32_t v[16];
+        ld16_issue(tE + tlane + (uint32_t)c_lo, v);
+#pragma unroll 1
+        for (int c0 = c_lo; c0 < c_lo + 64; c0 += 16) {
+          float d[16];
           const float4 y4[4] = {*reinterpret_cast<const float4 *>(yt + c0),
                                 *reinterpret_cast<const float4 *>(yt + c0 + 4),
                                 *reinterpret_cast<const float4 *>(yt + c0 + 8),
                                 *reinterpret_cast<const float4 *>(yt + c0 + 12)};
           const float *yy = reinterpret_cast<const float *>(y4);
-          float ls = 0.f;
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            float l = 0.f;
-            d[e] = 0.f;
-            if (fast || (live && t0 + c0 + e < r1)) fam_terms<FAM>(v[e], yy[e], inv_s2, nu, l, d[e]);
-            ls += l;
+          uint32_t okc = 0xFFFFu;
+          if (!fast) {
+            const int64_t left = r1 - (t0 + c0);
+            okc = !live || left <= 0 ? 0u : left >= 16 ? 0xFFFFu : (1u << left) - 1u;
           }
-          lsum += (double)ls;
+          uint32_t w[16];
+          ld16_wait(v);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) w[e] = v[e];
+          if (c0 + 16 < c_lo + 64) ld16_issue(tE + tlane + (uint32_t)(c0 + 16), v);
+          lsum += (double)fam_chunk<FAM>(w, yy, inv_s2, nu, okc, d);
           uint4 hi0, lo0, hi1, lo1;
           split8(d, hi0, lo0);
           split8(d + 8, hi1, lo1);
