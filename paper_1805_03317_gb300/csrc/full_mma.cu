@@ -155,8 +155,9 @@ __device__ __forceinline__ void fam_terms(float eta, float y, float inv_s2, floa
   }
 }
 
-// l and l' of 16 columns (d) and their sum of l. ok: bit e = column e counts.
-template <int FAM>
+// l and l' of 16 columns (d) and their sum of l. MASK: bit e of ok = column e counts (the last row and
+// particle tiles only: as selects the masks cost as much as the terms).
+template <int FAM, bool MASK>
 __device__ __forceinline__ float fam_chunk(const uint32_t (&v)[16], const float *y, float inv_s2,
                                            float nu, uint32_t ok, float (&d)[16]) {
   if constexpr (FAM == 0) {
@@ -178,7 +179,7 @@ __device__ __forceinline__ float fam_chunk(const uint32_t (&v)[16], const float 
       const float2 om = __ffma2_rn(s, mone, one);
       float2 mm = make_float2(fmaxf(s.x, om.x), fmaxf(s.y, om.y));
       float2 a = __ffma2_rn(ye, et, make_float2(fminf(-et.x, 0.f), fminf(-et.y, 0.f)));
-      if (ok != 0xFFFFu) {
+      if (MASK) {
         if (!(ok >> e & 1u)) dd.x = a.x = 0.f, mm.x = 1.f;
         if (!(ok >> (e + 1) & 1u)) dd.y = a.y = 0.f, mm.y = 1.f;
       }
@@ -194,7 +195,7 @@ __device__ __forceinline__ float fam_chunk(const uint32_t (&v)[16], const float 
     for (int e = 0; e < 16; ++e) {
       float l = 0.f;
       d[e] = 0.f;
-      if (ok >> e & 1u) fam_terms<FAM>(__uint_as_float(v[e]), y[e], inv_s2, nu, l, d[e]);
+      if (!MASK || (ok >> e & 1u)) fam_terms<FAM>(__uint_as_float(v[e]), y[e], inv_s2, nu, l, d[e]);
       ls += l;
     }
     return ls;
@@ -358,27 +359,28 @@ __global__ void __launch_bounds__(kThreads) k_full_mma(
         const float *yt = ys + b * kR;
         const bool fast = full_p && t0 + kR <= r1;
         const int c_lo = half * 64;
-        uint32_t v[16];
-        ld16_issue(tE + tlane + (uint32_t)c_lo, v);
-#pragma unroll 1
-        for (int c0 = c_lo; c0 < c_lo + 64; c0 += 16) {
+        uint32_t v[2][16];
+        ld16_issue(tE + tlane + (uint32_t)c_lo, v[0]);
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+          const int c0 = c_lo + 16 * ch;
           float d[16];
           const float4 y4[4] = {*reinterpret_cast<const float4 *>(yt + c0),
                                 *reinterpret_cast<const float4 *>(yt + c0 + 4),
                                 *reinterpret_cast<const float4 *>(yt + c0 + 8),
                                 *reinterpret_cast<const float4 *>(yt + c0 + 12)};
           const float *yy = reinterpret_cast<const float *>(y4);
-          uint32_t okc = 0xFFFFu;
-          if (!fast) {
+          ld16_wait(v[ch & 1]);
+          if (ch < 3) ld16_issue(tE + tlane + (uint32_t)(c0 + 16), v[(ch + 1) & 1]);
+          float ls;
+          if (fast) {
+            ls = fam_chunk<FAM, false>(v[ch & 1], yy, inv_s2, nu, 0u, d);
+          } else {
             const int64_t left = r1 - (t0 + c0);
-            okc = !live || left <= 0 ? 0u : left >= 16 ? 0xFFFFu : (1u << left) - 1u;
+            const uint32_t ok = !live || left <= 0 ? 0u : left >= 16 ? 0xFFFFu : (1u << left) - 1u;
+            ls = fam_chunk<FAM, true>(v[ch & 1], yy, inv_s2, nu, ok, d);
           }
-          uint32_t w[16];
-          ld16_wait(v);
-#pragma unroll
-          for (int e = 0; e < 16; ++e) w[e] = v[e];
-          if (c0 + 16 < c_lo + 64) ld16_issue(tE + tlane + (uint32_t)(c0 + 16), v);
-          lsum += (double)fam_chunk<FAM>(w, yy, inv_s2, nu, okc, d);
+          lsum += (double)ls;
           uint4 hi0, lo0, hi1, lo1;
           split8(d, hi0, lo0);
           split8(d + 8, hi1, lo1);
