@@ -19,6 +19,8 @@
 // sums per block: sum d = sum e + n_g K, sum d^2 = sum e^2 + 2 K sum e + n_g K^2.
 #pragma once
 
+#include <type_traits>
+
 #include "device.cuh"
 #include "internal.h"
 
@@ -63,6 +65,12 @@ template <typename CT> struct RowIO {
 // barrier. (When the tiles' chunks end before the tail, the owner copies its tail itself.)
 // Chunk vectors are XOR-swizzled so that 128-bit reads of 8 consecutive lanes hit distinct bank
 // groups; chunk vectors that lie past the covariates are never copied and stay zero.
+// First row of block g of the floor partition of m rows into G blocks (g <= G <= m < 2^31).
+__device__ __forceinline__ int block_first(int g, int m, int G) {
+  const uint64_t v = (uint64_t)(uint32_t)g * (uint32_t)m;
+  return (v >> 32) ? (int)(v / (uint32_t)G) : (int)((uint32_t)v / (uint32_t)G);
+}
+
 template <typename XT, int T, int CPL, int NST, bool PIPE = false>
 struct WarpEval {
   using SD = Store<XT>;
@@ -127,8 +135,8 @@ struct WarpEval {
 
   // One pass over rows idx[0..nrows). GRAD: accumulates the gradient partials sum r x, sum d r x
   // over this lane's slots into g1, g2. Returns S = sum d and Q = sum d^2 on every lane; BLOCKS
-  // also writes per-block (sum d, sum d^2) of the floor partition of the nrows rows into G blocks
-  // to blk_out[2G].
+  // also writes per-block (sum d, sum d^2) to blk_out[2G]: the rows are whole blocks, from block
+  // g_first on, of the floor partition of mtot rows into G blocks.
   // The sums are of e = d - K (returned in Ksh, warp-uniform: the d of row 0), so
   // Ssum = sum e and Qsum = sum e^2; g2 accumulates e r x. BLOCKS writes the unshifted FP64 block
   // sums (sum d, sum d^2) rebuilt from the shifted ones.
@@ -137,7 +145,8 @@ struct WarpEval {
                                        const int32_t *idx, int nrows, int fam, CT inv_s2, CT *g1,
                                        CT *g2, double *blk_out, int G, double &Ssum, double &Qsum,
                                        double &Ksh, DevState *st,
-                                       const RowIO<CT> &io = RowIO<CT>(), int cv1 = 0) const {
+                                       const RowIO<CT> &io = RowIO<CT>(), int cv1 = 0,
+                                       int g_first = 0, int mtot = 0) const {
     const int nsw = (nrows + 31) >> 5;
     // rows past the end copy the last row again (already on chip) and are masked out
     const int klast = nrows > 0 ? idx[nrows - 1] : 0;
@@ -185,22 +194,35 @@ struct WarpEval {
       }
       cp_async_commit();  // one group per sweep (empty past the end) keeps the counting uniform
     };
-    if (BLOCKS) {
-      for (int h = lane; h < 2 * G; h += 32) blk_out[h] = 0.0;  // blocks with no rows stay zero
-      __syncwarp();
-    }
-    CT sd = CT(0), sd2 = CT(0);
-    double cs = 0.0, cq = 0.0;  // BLOCKS: shifted sums of the open block cg
-    int cg = -1;
+    CT sd = CT(0), sd2 = CT(0);  // lane sums of e, e^2 (BLOCKS: of the open block since its last flush)
     CT K = CT(0);               // shift of the sums: d of row 0 (set at sweep 0)
     Ssum = Qsum = 0.0;
-    // close block g: its unshifted FP64 sums from the shifted ones
-    auto close_block = [&](int g) {
-      const double ng = (double)((int)(((int64_t)(g + 1) * nrows) / G) -
-                                 (int)(((int64_t)g * nrows) / G));
-      const double k = (double)K;
-      blk_out[2 * g] = fma(ng, k, cs);
-      blk_out[2 * g + 1] = cq + k * fma(ng, k, 2.0 * cs);
+    // BLOCKS: the open block cg, local rows up to jend, and what its flushes have summed
+    int cg = g_first, nfl = 0;
+    const int j0g = BLOCKS ? block_first(g_first, mtot, G) : 0;
+    int jend = BLOCKS ? block_first(cg + 1, mtot, G) - j0g : 0;
+    double cs = 0.0, cq = 0.0;
+    constexpr bool EACH = sizeof(CT) == 8;  // FP64 rows: a sum per sweep (their terms dominate)
+    auto flush = [&]() {
+      const CT bs = warp_sum(sd), bq = warp_sum(sd2);
+      if (EACH) {
+        Ssum += (double)bs;
+        Qsum += (double)bq;
+      }
+      cs = nfl ? cs + (double)bs : (double)bs;
+      cq = nfl ? cq + (double)bq : (double)bq;
+      ++nfl;
+      sd = sd2 = CT(0);
+    };
+    auto close_block = [&]() {
+      flush();
+      if (lane == 0) {
+        blk_out[2 * cg] = cs;
+        blk_out[2 * cg + 1] = cq;
+      }
+      nfl = 0;
+      ++cg;
+      jend = block_first(cg + 1, mtot, G) - j0g;
     };
     // partial x'delta of the group's T rows over this lane's slots, reduce-scattered: the full D of
     // the row this lane owns
@@ -253,25 +275,24 @@ struct WarpEval {
       }
       if (s == 0) K = __shfl_sync(0xffffffffu, d, 0);  // every lane is here at sweep 0
       d = valid ? d - K : CT(0);  // from here on d holds e = d - K
-      if (BLOCKS) {  // block of row j: largest g with floor(g nrows / G) <= j
-        const int r1 = min((s << 5) + 31, nrows - 1);
-        const int gA = (int)(((unsigned)((s << 5) + 1) * (unsigned)G - 1u) / (unsigned)nrows);
-        const int gB = (int)(((unsigned)(r1 + 1) * (unsigned)G - 1u) / (unsigned)nrows);
-        const int gj =
-            j < nrows ? (int)(((unsigned)(j + 1) * (unsigned)G - 1u) / (unsigned)nrows) : -1;
-        for (int g = gA; g <= gB; ++g) {
-          const CT bs = warp_sum(gj == g ? d : CT(0));
-          const CT bq = warp_sum(gj == g ? d * d : CT(0));
-          if (g != cg) {
-            if (cg >= 0 && lane == 0) close_block(cg);
-            cg = g;
-            cs = cq = 0.0;
+      if (BLOCKS) {
+        // Lane sums within a block, flushed through a warp tree into FP64 when the block closes (or
+        // after 8 sweeps): an FP64 add holds the warp's pipe for 64 cycles, so not one per sweep
+        // (1000 rows, 10 blocks: 123 us for 4096 particles with sums per sweep, 84 us now).
+        int rest = 0;  // rows of the sweep before this one belong to closed blocks
+        while (jend <= min((s << 5) + 32, nrows)) {  // (no block is empty: G <= m)
+          if (j >= rest && j < jend) {
+            sd += d;
+            sd2 = fma(d, d, sd2);
           }
-          cs += (double)bs;
-          cq += (double)bq;
-          Ssum += (double)bs;
-          Qsum += (double)bq;
+          rest = jend;
+          close_block();
         }
+        if (j >= rest && j < nrows) {
+          sd += d;
+          sd2 = fma(d, d, sd2);
+        }
+        if (EACH ? jend > min((s << 5) + 32, nrows) && rest < nrows : (s & 7) == 7) flush();
       } else {
         sd += d;
         sd2 = fma(d, d, sd2);
@@ -341,15 +362,31 @@ struct WarpEval {
       }
     }
     cp_async_wait<0>();
+    Ksh = (double)K;
     if (BLOCKS) {
-      if (cg >= 0 && lane == 0) close_block(cg);
+      // totals, and the blocks' unshifted FP64 sums from the shifted ones, one block per lane
+      __syncwarp();
+      for (int g = g_first + lane; g < cg; g += 32) {
+        const double ng = (double)(block_first(g + 1, mtot, G) - block_first(g, mtot, G));
+        const double se = blk_out[2 * g], qe = blk_out[2 * g + 1];
+        if (!EACH) {
+          Ssum += se;
+          Qsum += qe;
+        }
+        blk_out[2 * g] = fma(ng, Ksh, se);
+        blk_out[2 * g + 1] = qe + Ksh * fma(ng, Ksh, 2.0 * se);
+      }
+      if (!EACH) {
+        Ssum = warp_sum(Ssum);
+        Qsum = warp_sum(Qsum);
+      }
     } else {
       Ssum = warp_sum((double)sd);
       Qsum = warp_sum((double)sd2);
     }
-    Ksh = (double)K;
   }
 };
+
 
 // Shared-memory scratch of one warp: theta, delta, rho, grad, v [p each] and the reduced gradient
 // partials G1, G2 [T*CPL each], all in the state type.
@@ -379,16 +416,34 @@ template <typename CT> __device__ __forceinline__ CT ldg_ct(const void *p, int i
   return __ldg(reinterpret_cast<const CT *>(p) + i);
 }
 
-// One evaluation of the estimator for the warp's particle at theta (in sm.th / sm.dl).
-// Reads rows of idx[0..m); GRAD: writes the target gradient to sm.g; BLOCKS: writes per-block
-// (sum d, sum d^2) to blk_out[G*2]. Returns l_hat and sigma2_hat on every lane.
-template <typename XT, int T, int CPL, int U, bool K, bool GRAD, bool BLOCKS, int MODE = 0>
-__device__ __forceinline__ void eval_particle(const WarpEval<XT, T, CPL, U, K> &W, const EstArgs &a,
+// The rows of a particle that warp w of a CTA takes when the CTA's W warps share one particle: whole
+// sweeps, or whole blocks where the block sums are wanted. j0, j1: the rows; g0: their first block.
+__device__ __forceinline__ void split_rows(int m, int G, int w, int W, bool blocks, int &j0, int &j1,
+                                           int &g0) {
+  // parts rounded up, so that the first warp is never without rows (its shift is the merge's)
+  const int n = blocks ? G : (m + 31) >> 5;
+  const int p0 = (int)(((int64_t)w * n + W - 1) / W), p1 = (int)(((int64_t)(w + 1) * n + W - 1) / W);
+  g0 = blocks ? p0 : 0;
+  j0 = blocks ? block_first(p0, m, G) : 32 * p0;
+  j1 = blocks ? block_first(p1, m, G) : 32 * p1;
+  j0 = min(j0, m);
+  j1 = min(j1, m);
+}
+
+// One evaluation of the estimator for a particle at theta (in sm.th / sm.dl) by one warp, or, with
+// SPLIT > 1, by the SPLIT warps of its CTA (warp `part` this one; each has its own sm, `stride` bytes
+// apart): every warp sums its own rows, and warp 0 merges them. Returns whether this warp is the one
+// that holds the result. Reads rows of idx[0..m); GRAD: writes the target gradient to sm.g; BLOCKS:
+// writes per-block (sum d, sum d^2) to blk_out[G*2]. l_hat and sigma2_hat on every lane.
+template <typename XT, int T, int CPL, int U, bool K, bool GRAD, bool BLOCKS, int MODE = 0,
+          int SPLIT = 1>
+__device__ __forceinline__ bool eval_particle(const WarpEval<XT, T, CPL, U, K> &W, const EstArgs &a,
                                               const int32_t *idx, WarpSmem<typename Store<XT>::CT> &sm,
                                               double temp, double *blk_out, double &ell,
                                               double &sig2,
-                                              const RowIO<typename Store<XT>::CT> &io =
-                                                  RowIO<typename Store<XT>::CT>()) {
+                                              const RowIO<typename Store<XT>::CT> &io_ =
+                                                  RowIO<typename Store<XT>::CT>(),
+                                              int part = 0, int stride = 0) {
   using CT = typename Store<XT>::CT;
   const XT *Xp = reinterpret_cast<const XT *>(a.Xp);
   const CT inv_s2 = (CT)a.inv_s2;
@@ -396,10 +451,18 @@ __device__ __forceinline__ void eval_particle(const WarpEval<XT, T, CPL, U, K> &
 #pragma unroll
   for (int s = 0; s < CPL; ++s) g1[s] = g2[s] = CT(0);
   double S, Q, Ks;  // sums of e = d - Ks and e^2, and the shift Ks
-  W.template rows<GRAD, BLOCKS, MODE>(Xp, a.S, a.n, idx, a.m, a.fam, inv_s2, g1, g2, blk_out, a.G,
-                                      S, Q, Ks, a.st, io, a.cv_order == 1);
+  int j0 = 0, j1 = a.m, gb0 = 0;
+  RowIO<CT> io = io_;
+  if constexpr (SPLIT > 1) {
+    split_rows(a.m, a.G, part, SPLIT, BLOCKS, j0, j1, gb0);
+    if (MODE == 1) {
+      io.dsave += j0;
+      io.rsave += j0;
+    }
+  }
+  W.template rows<GRAD, BLOCKS, MODE>(Xp, a.S, a.n, idx + j0, j1 - j0, a.fam, inv_s2, g1, g2,
+                                      blk_out, a.G, S, Q, Ks, a.st, io, a.cv_order == 1, gb0, a.m);
   const double nm = (double)a.n / (double)a.m;
-  const double dbar = S / (double)a.m;  // mean of e (the gradient partials hold e r x)
   if (GRAD) {
     // reduce the gradient partials over the row slots of the warp
 #pragma unroll
@@ -419,6 +482,35 @@ __device__ __forceinline__ void eval_particle(const WarpEval<XT, T, CPL, U, K> &
     }
   }
   __syncwarp();
+  if constexpr (SPLIT > 1) {
+    // merge: sums about the first warp's shift, S = sum_w (S_w + n_w k_w) and Q = sum_w (Q_w +
+    // k_w (2 S_w + n_w k_w)) with k_w = K_w - K_0 (Chan, Golub & LeVeque 1983), and the gradient
+    // partials' sum e r x likewise
+    __shared__ double merge[8][4];
+    if (W.lane == 0) {
+      merge[part][0] = S;
+      merge[part][1] = Q;
+      merge[part][2] = Ks;
+      merge[part][3] = (double)(j1 - j0);
+    }
+    __syncthreads();
+    if (part) return false;
+    for (int w = 1; w < SPLIT; ++w) {
+      const double nw = merge[w][3], k = nw > 0.0 ? merge[w][2] - Ks : 0.0;
+      S += fma(nw, k, merge[w][0]);
+      Q += merge[w][1] + k * fma(nw, k, 2.0 * merge[w][0]);
+      if (GRAD) {
+        const CT kc = (CT)k;
+        const int off = w * stride / (int)sizeof(CT);
+        for (int c = W.lane; c < a.p; c += 32) {
+          const CT h1 = sm.G1[c + off];
+          sm.G1[c] += h1;
+          sm.G2[c] += fma(kc, h1, sm.G2[c + off]);
+        }
+      }
+    }
+  }
+  const double dbar = S / (double)a.m;  // mean of e (the gradient partials hold e r x)
   // delta'(B + C delta / 2) and, with GRAD, the per-column gradient
   const int p = a.p;
   double qlin = 0.0;
@@ -439,6 +531,7 @@ __device__ __forceinline__ void eval_particle(const WarpEval<XT, T, CPL, U, K> &
   ell = (a.A_dev ? __ldg(a.A_dev) : a.A) + qlin + nm * fma((double)a.m, Ks, S);
   sig2 = nm * nm * fmax(0.0, Q - S * S / (double)a.m);
   __syncwarp();
+  return true;
 }
 
 template <typename CT> __device__ __forceinline__ double log_prior_warp(const EstArgs &a,
@@ -477,16 +570,23 @@ __device__ __forceinline__ int batch_problem(const int *offsets, int nprob, int 
 // ------------------------------------------------------------------------------------------------
 // Kernel 1: the plain estimator on caller particles (loglik_est / loglik_grad, cache refresh).
 // ------------------------------------------------------------------------------------------------
-template <typename XT, int T, int CPL, int U, int WARPS, bool K>
+// SPLIT = WARPS: one CTA per particle, its warps sharing the rows (few particles); 1: one warp each.
+// USE: one kernel per use, so that its sweep loop has the instruction cache and the registers to itself
+// (the cache refresh of the 2 x 16-slot tile needs 64 registers instead of 123: 4096 particles of
+// m = 1000, p = 20, 122 us before). kUseAny, chosen by a.grad and a.blk, serves the gradient of the
+// tiles with eight lanes per row or more, whose schedule in a kernel of its own was slower (p = 101,
+// 16384 particles of m = 5000: 3.67 ms against 3.87; p = 50 with four lanes: 403 against 383 us).
+enum EstUse { kUseEst = 0, kUseGrad = 1, kUseCache = 2, kUseAny = 3 };
+template <typename XT, int T, int CPL, int U, int WARPS, bool K, int SPLIT, int USE>
 __global__ void __launch_bounds__(WARPS * 32) k_estimate(EstArgs a) {
   using CT = typename Store<XT>::CT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * WARPS + warp;
-  if (i >= a.B) return;  // whole warp leaves together; no block-level barriers follow
+  const int i = SPLIT > 1 ? blockIdx.x : blockIdx.x * WARPS + warp;
+  if (i >= a.B) return;  // whole warp leaves together; without SPLIT no block-level barriers follow
   WarpEval<XT, T, CPL, U, K> W;
-  const int slots = T * CPL;
-  unsigned char *wbase = smem_raw + (size_t)warp * warp_smem_bytes<XT, T, CPL, U>(a.p);
+  const int slots = T * CPL, stride = warp_smem_bytes<XT, T, CPL, U>(a.p);
+  unsigned char *wbase = smem_raw + (size_t)warp * stride;
   W.init(wbase, a.Yo);
   WarpSmem<CT> sm(reinterpret_cast<CT *>(wbase + WarpEval<XT, T, CPL, U, K>::RING), a.p, slots);
   const CT *th = reinterpret_cast<const CT *>(a.theta) + (int64_t)i * a.p;
@@ -496,19 +596,31 @@ __global__ void __launch_bounds__(WARPS * 32) k_estimate(EstArgs a) {
   const double temp = a.a_from_state ? a.st->a : a.a_host;
   const int32_t *idx = a.u + (int64_t)i * a.m;
   double ell, sig2;
-  double *blk = a.blk ? a.blk + (int64_t)i * a.G * 2 : nullptr;
-  if (a.grad) {
-    if (blk)
-      eval_particle<XT, T, CPL, U, K, true, true>(W, a, idx, sm, temp, blk, ell, sig2);
-    else
-      eval_particle<XT, T, CPL, U, K, true, false>(W, a, idx, sm, temp, nullptr, ell, sig2);
-    CT *g = reinterpret_cast<CT *>(a.grad) + (int64_t)i * a.p;
-    for (int c = W.lane; c < a.p; c += 32) g[c] = sm.g[c];
+  if constexpr (USE == kUseAny) {
+    double *blk = a.blk ? a.blk + (int64_t)i * a.G * 2 : nullptr;
+    const RowIO<CT> io;
+    auto eval = [&](auto grad_c, auto blocks_c) {
+      return eval_particle<XT, T, CPL, U, K, decltype(grad_c)::value, decltype(blocks_c)::value, 0,
+                           SPLIT>(W, a, idx, sm, temp, blk, ell, sig2, io, warp, stride);
+    };
+    constexpr std::true_type yes{};
+    constexpr std::false_type no{};
+    if (!(a.grad ? (blk ? eval(yes, yes) : eval(yes, no)) : (blk ? eval(no, yes) : eval(no, no))))
+      return;
+    if (a.grad) {
+      CT *g = reinterpret_cast<CT *>(a.grad) + (int64_t)i * a.p;
+      for (int c = W.lane; c < a.p; c += 32) g[c] = sm.g[c];
+    }
   } else {
-    if (blk)
-      eval_particle<XT, T, CPL, U, K, false, true>(W, a, idx, sm, temp, blk, ell, sig2);
-    else
-      eval_particle<XT, T, CPL, U, K, false, false>(W, a, idx, sm, temp, nullptr, ell, sig2);
+    constexpr bool GRAD = USE == kUseGrad, BLOCKS = USE == kUseCache;
+    double *blk = BLOCKS ? a.blk + (int64_t)i * a.G * 2 : nullptr;
+    if (!eval_particle<XT, T, CPL, U, K, GRAD, BLOCKS, 0, SPLIT>(W, a, idx, sm, temp, blk, ell,
+                                                                 sig2, RowIO<CT>(), warp, stride))
+      return;
+    if (GRAD) {
+      CT *g = reinterpret_cast<CT *>(a.grad) + (int64_t)i * a.p;
+      for (int c = W.lane; c < a.p; c += 32) g[c] = sm.g[c];
+    }
   }
   if (W.lane == 0) {
     if (a.ell) a.ell[i] = ell;
@@ -524,15 +636,16 @@ __global__ void __launch_bounds__(WARPS * 32) k_estimate(EstArgs a) {
 //   dL/dtheta = g_l (B + C delta) + sum_j r_j [g_l n/m + g_s 2 (n/m)^2 (d_j - dbar)] x_j
 // from the saved values and the rows gathered again by u (no family terms are re-evaluated).
 // ------------------------------------------------------------------------------------------------
-template <typename XT, int T, int CPL, int U, int WARPS, bool K>
+template <typename XT, int T, int CPL, int U, int WARPS, bool K, int SPLIT>
 __global__ void __launch_bounds__(WARPS * 32) k_fwdsave(EstArgs a) {
   using CT = typename Store<XT>::CT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * WARPS + warp;
+  const int i = SPLIT > 1 ? blockIdx.x : blockIdx.x * WARPS + warp;
   if (i >= a.B) return;
   WarpEval<XT, T, CPL, U, K> W;
-  unsigned char *wbase = smem_raw + (size_t)warp * warp_smem_bytes<XT, T, CPL, U>(a.p);
+  const int stride = warp_smem_bytes<XT, T, CPL, U>(a.p);
+  unsigned char *wbase = smem_raw + (size_t)warp * stride;
   W.init(wbase, a.Yo);
   WarpSmem<CT> sm(reinterpret_cast<CT *>(wbase + WarpEval<XT, T, CPL, U, K>::RING), a.p, T * CPL);
   const CT *th = reinterpret_cast<const CT *>(a.theta) + (int64_t)i * a.p;
@@ -543,8 +656,10 @@ __global__ void __launch_bounds__(WARPS * 32) k_fwdsave(EstArgs a) {
   io.dsave = reinterpret_cast<CT *>(a.dsave) + (int64_t)i * a.m;
   io.rsave = reinterpret_cast<CT *>(a.rsave) + (int64_t)i * a.m;
   double ell, sig2;
-  eval_particle<XT, T, CPL, U, K, false, false, 1>(W, a, a.u + (int64_t)i * a.m, sm, 1.0, nullptr,
-                                                    ell, sig2, io);
+  if (!eval_particle<XT, T, CPL, U, K, false, false, 1, SPLIT>(W, a, a.u + (int64_t)i * a.m, sm,
+                                                                1.0, nullptr, ell, sig2, io, warp,
+                                                                stride))
+    return;
   if (W.lane == 0) {
     a.ell[i] = ell;
     a.sig2[i] = sig2;
@@ -552,16 +667,16 @@ __global__ void __launch_bounds__(WARPS * 32) k_fwdsave(EstArgs a) {
   }
 }
 
-template <typename XT, int T, int CPL, int U, int WARPS, bool K>
+template <typename XT, int T, int CPL, int U, int WARPS, bool K, int SPLIT>
 __global__ void __launch_bounds__(WARPS * 32) k_backward(EstArgs a) {
   using CT = typename Store<XT>::CT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * WARPS + warp;
+  const int i = SPLIT > 1 ? blockIdx.x : blockIdx.x * WARPS + warp;
   if (i >= a.B) return;
   WarpEval<XT, T, CPL, U, K> W;
-  const int p = a.p, m = a.m;
-  unsigned char *wbase = smem_raw + (size_t)warp * warp_smem_bytes<XT, T, CPL, U>(p);
+  const int p = a.p, m = a.m, stride = warp_smem_bytes<XT, T, CPL, U>(p);
+  unsigned char *wbase = smem_raw + (size_t)warp * stride;
   W.init(wbase, a.Yo);
   WarpSmem<CT> sm(reinterpret_cast<CT *>(wbase + WarpEval<XT, T, CPL, U, K>::RING), p, T * CPL);
   const CT *th = reinterpret_cast<const CT *>(a.theta) + (int64_t)i * p;
@@ -582,9 +697,15 @@ __global__ void __launch_bounds__(WARPS * 32) k_backward(EstArgs a) {
 #pragma unroll
   for (int e = 0; e < CPL; ++e) g1[e] = g2[e] = CT(0);
   double S_, Q_, K_;
+  int j0 = 0, j1 = m, gb0 = 0;
+  if constexpr (SPLIT > 1) {
+    split_rows(m, a.G, warp, WARPS, false, j0, j1, gb0);
+    io.dsaved += j0;
+    io.rsaved += j0;
+  }
   W.template rows<true, false, 2>(reinterpret_cast<const XT *>(a.Xp), a.S, a.n,
-                                  a.u + (int64_t)i * m, m, a.fam, (CT)a.inv_s2, g1, g2, nullptr,
-                                  a.G, S_, Q_, K_, a.st, io);
+                                  a.u + (int64_t)i * m + j0, j1 - j0, a.fam, (CT)a.inv_s2, g1, g2,
+                                  nullptr, a.G, S_, Q_, K_, a.st, io);
 #pragma unroll
   for (int e = 0; e < CPL; ++e) {
 #pragma unroll
@@ -595,6 +716,12 @@ __global__ void __launch_bounds__(WARPS * 32) k_backward(EstArgs a) {
     for (int e = 0; e < CPL; ++e) sm.G1[W.gl * CPL + e] = g1[e];
   }
   __syncwarp();
+  if constexpr (SPLIT > 1) {
+    __syncthreads();
+    if (warp) return;
+    for (int w = 1; w < WARPS; ++w)
+      for (int c = W.lane; c < p; c += 32) sm.G1[c] += sm.G1[c + w * stride / (int)sizeof(CT)];
+  }
   CT *gout = reinterpret_cast<CT *>(a.grad) + (int64_t)i * p;
   const CT cgl = (CT)gl;
   for (int c = W.lane; c < p; c += 32) {
@@ -602,6 +729,15 @@ __global__ void __launch_bounds__(WARPS * 32) k_backward(EstArgs a) {
     for (int k = 0; k < p; ++k) cd = fma(ldg_ct<CT>(a.C_ct, k * p + c), sm.dl[k], cd);
     gout[c] = cgl * (ldg_ct<CT>(a.B_ct, c) + cd) + sm.G1[c];
   }
+}
+
+// log U < t for U in [0, 1). The FP32 logarithm decides unless it lies within 1e-3 of t (its error is
+// below 1e-5: |log U| <= 37, a few units in the last place), where the FP64 one does: the same
+// decisions, without some 40 FP64 instructions of 64 pipe cycles each for almost every particle.
+__device__ __forceinline__ bool log_below(double U, double t) {
+  const double d = (double)logf((float)U) - t;
+  if (fabs(d) > 1e-3) return d < 0.0;  // (U = 0: -inf; a NaN t goes on)
+  return log(U) < t;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -659,8 +795,7 @@ __device__ __forceinline__ void upm_body(const EstArgs &a, int i, unsigned char 
   const double sig1 = nm * nm * fmax(0.0, Qn - Sn * Sn / (double)a.m);
   const double log_r = temp * (ell1 - ell0) - 0.5 * temp * temp * (sig1 - sig0);
   const Stream smh(a.seed, kMhU, smv, (uint32_t)i);
-  const double Uu = draw_uniform(smh.draw(0));
-  const bool acc = log(Uu) < log_r;
+  const bool acc = log_below(draw_uniform(smh.draw(0)), log_r);
   if (acc) {
     int32_t *ui = a.u_mut + (int64_t)i * a.m + j0;
     for (int t = W.lane; t < nb; t += 32) ui[t] = unew[t];
@@ -845,33 +980,51 @@ __global__ void __launch_bounds__(WARPS * 32) k_hmc_batch(BatchArgs b) {
 // ------------------------------------------------------------------------------------------------
 // Launch helpers
 // ------------------------------------------------------------------------------------------------
+// Particles up to which a CTA's warps share one particle in the estimator kernels: beyond, one warp
+// per particle fills the GPU better than four that repeat the work per particle. us with one warp /
+// shared, gradient: logistic BF16 p = 20, m = 1000: 32 / 23 for 280 particles, 32 / 26 for 608,
+// 37 / 42 for 1000; Student-t p = 50, m = 1250: 47 / 31, 49 / 35, 62 / 61; FP64 p = 5, m = 100:
+// 37 / 31, 38 / 47, 62 / 82.
+template <typename CT> constexpr int kSplitParticles = (sizeof(CT) == 8 ? 2 : 4) * 152;
+
 template <typename XT, int T, int CPL, int U, int WARPS, bool K = false>
 inline int launch_tile(int op, const EstArgs &a, cudaStream_t s) {
-  using CT = typename Store<XT>::CT;
   const size_t smem = (size_t)WARPS * warp_smem_bytes<XT, T, CPL, U>(a.p);
-  const dim3 grid((a.B + WARPS - 1) / WARPS), block(WARPS * 32);
   if (a.B <= 0) return 0;
-  cudaError_t e;
+  // (the cache of FP64 states keeps one summation order for every N)
+  const bool split = WARPS > 1 && (op == 0 || op >= 3) && a.B <= kSplitParticles<typename Store<XT>::CT> &&
+                     !(sizeof(XT) == 8 && a.blk);
+  const dim3 grid(split ? a.B : (a.B + WARPS - 1) / WARPS), block(WARPS * 32);
+  cudaError_t e = cudaSuccess;
+  auto go = [&](auto *kernel) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) kernel<<<grid, block, smem, s>>>(a);
+  };
   if (op == 0) {
-    e = cudaFuncSetAttribute(k_estimate<XT, T, CPL, U, WARPS, K>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) k_estimate<XT, T, CPL, U, WARPS, K><<<grid, block, smem, s>>>(a);
+    constexpr int kGrad = T >= 8 ? kUseAny : kUseGrad;
+    if (a.grad && a.blk) return (int)cudaErrorInvalidValue;  // (no entry point asks for both)
+    if (split)
+      a.grad  ? go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, kUseGrad>)
+      : a.blk ? go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, kUseCache>)
+              : go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, kUseEst>);
+    else
+      a.grad  ? go(k_estimate<XT, T, CPL, U, WARPS, K, 1, kGrad>)
+      : a.blk ? go(k_estimate<XT, T, CPL, U, WARPS, K, 1, kUseCache>)
+              : go(k_estimate<XT, T, CPL, U, WARPS, K, 1, kUseEst>);
   } else if (op == 1) {
-    e = cudaFuncSetAttribute(k_upm<XT, T, CPL, U, WARPS, K>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) k_upm<XT, T, CPL, U, WARPS, K><<<grid, block, smem, s>>>(a);
+    go(k_upm<XT, T, CPL, U, WARPS, K>);
   } else if (op == 2) {
-    e = cudaFuncSetAttribute(k_hmc<XT, T, CPL, U, WARPS, K>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) k_hmc<XT, T, CPL, U, WARPS, K><<<grid, block, smem, s>>>(a);
+    go(k_hmc<XT, T, CPL, U, WARPS, K>);
   } else if (op == 3) {
-    e = cudaFuncSetAttribute(k_fwdsave<XT, T, CPL, U, WARPS, K>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) k_fwdsave<XT, T, CPL, U, WARPS, K><<<grid, block, smem, s>>>(a);
+    if (split)
+      go(k_fwdsave<XT, T, CPL, U, WARPS, K, WARPS>);
+    else
+      go(k_fwdsave<XT, T, CPL, U, WARPS, K, 1>);
   } else {
-    e = cudaFuncSetAttribute(k_backward<XT, T, CPL, U, WARPS, K>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) k_backward<XT, T, CPL, U, WARPS, K><<<grid, block, smem, s>>>(a);
+    if (split)
+      go(k_backward<XT, T, CPL, U, WARPS, K, WARPS>);
+    else
+      go(k_backward<XT, T, CPL, U, WARPS, K, 1>);
   }
   if (e != cudaSuccess) return (int)e;
   return (int)cudaGetLastError();
