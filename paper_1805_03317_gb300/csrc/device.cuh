@@ -190,7 +190,11 @@ template <typename CT, int K0> __device__ __forceinline__ CT exp_tail(CT D) {
 }
 
 // log Phi(z) and lambda(z) = phi(z)/Phi(z) from CUDA's erfc/erfcx.
-template <typename CT> __device__ __forceinline__ void log_phi_(CT z, CT &lp, CT &lam) {
+// A translation unit may have it called instead of inlined (defined before this header is included).
+#ifndef SUBSMC_LOG_PHI_CALL
+#define SUBSMC_LOG_PHI_CALL __forceinline__
+#endif
+template <typename CT> __device__ SUBSMC_LOG_PHI_CALL void log_phi_(CT z, CT &lp, CT &lam) {
   const CT x = -z * CT(0.70710678118654752440);
   const CT ex = erfcx(x);
   lam = CT(0.79788456080286535588) / ex;
@@ -324,11 +328,8 @@ __device__ __forceinline__ void horner2<float>(float &pd, float &pr, float D, fl
   pr = v.y;
 }
 
-// short4: the caller has checked |D| <= 1/20 for every lane of the warp (FP32 only); the
-// logistic series then stops at kappa_6 (truncation below 2e-8 of w|D|^3 and w D^2).
 template <int FAM, typename CT>
-__device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT &d, CT &r,
-                                         bool short4 = false) {
+__device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT &d, CT &r) {
   if (FAM == 0) {  // logistic: l = y*eta - log(1 + e^eta); y cancels from d and r
     const CT sb = c.c0, w = c.c1;
     // With K(D) = log(1 - s + s e^D), the cumulant generating function of Bernoulli(s), s = sigma(eta_bar):
@@ -338,21 +339,6 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
     // relative error below 1e-8 in d and 1e-7 in r (1e-15 in FP64). No transcendental, no
     // division, no cancellation.
     constexpr CT kSmall = sizeof(CT) == 8 ? CT(0.05) : CT(0.5);
-    if (sizeof(CT) == 4 && short4) {
-      const CT q = CT(1) - CT(2) * sb;
-      const CT k3 = w * q;
-      const CT k4 = w * (CT(1) - CT(6) * w);
-      const CT k5 = k3 * (CT(1) - CT(12) * w);
-      const CT k6 = w * (CT(1) + w * (CT(-30) + CT(120) * w));
-      CT pd = k6 * CT(1.0 / 720.0), pr = k6 * CT(1.0 / 120.0);
-      horner2(pd, pr, D, k5, 1.0 / 120.0, 1.0 / 24.0);
-      horner2(pd, pr, D, k4, 1.0 / 24.0, 1.0 / 6.0);
-      horner2(pd, pr, D, k3, 1.0 / 6.0, 0.5);
-      const CT D2 = D * D;
-      d = -D2 * D * pd;
-      r = -D2 * pr;
-      return;
-    }
     // FP32: one form per warp (a vote over the lanes evaluating a row here), so a warp whose rows
     // straddle |D| = 1/2 does not run both forms; rows with small |D| in a warp that takes the
     // exp/log form carry that form's absolute error (about 3e-7) instead of the series' relative one

@@ -252,10 +252,8 @@ struct WarpEval {
         return;
       }
       const RowC<CT> c = *reinterpret_cast<const RowC<CT> *>(tail(b));
-      // every lane evaluates a row here, so a warp vote is safe
-      const bool short4 = __all_sync(0xffffffffu, fabs(D) <= CT(0.05));
       switch (fam) {
-        case 0: row_incr<0, CT>(c, D, inv_s2, d, r, short4); break;
+        case 0: row_incr<0, CT>(c, D, inv_s2, d, r); break;
         case 1: row_incr<1, CT>(c, D, inv_s2, d, r); break;
         case 2: row_incr<2, CT>(c, D, inv_s2, d, r); break;
         case 3: row_incr<3, CT>(c, D, inv_s2, d, r); break;
@@ -571,13 +569,10 @@ __device__ __forceinline__ int batch_problem(const int *offsets, int nprob, int 
 // Kernel 1: the plain estimator on caller particles (loglik_est / loglik_grad, cache refresh).
 // ------------------------------------------------------------------------------------------------
 // SPLIT = WARPS: one CTA per particle, its warps sharing the rows (few particles); 1: one warp each.
-// USE: one kernel per use, so that its sweep loop has the instruction cache and the registers to itself
-// (the cache refresh of the 2 x 16-slot tile needs 64 registers instead of 123: 4096 particles of
-// m = 1000, p = 20, 122 us before). kUseAny, chosen by a.grad and a.blk, serves the gradient of the
-// tiles with eight lanes per row or more, whose schedule in a kernel of its own was slower (p = 101,
-// 16384 particles of m = 5000: 3.67 ms against 3.87; p = 50 with four lanes: 403 against 383 us).
-enum EstUse { kUseEst = 0, kUseGrad = 1, kUseCache = 2, kUseAny = 3 };
-template <typename XT, int T, int CPL, int U, int WARPS, bool K, int SPLIT, int USE>
+// GRAD: with the gradient (a.grad); BLOCKS: with the block sums (a.blk). One kernel per use, so that
+// its sweep loop has the instruction cache and the registers to itself (the cache refresh of the
+// 2 x 16-slot tile needs 64 registers instead of 123).
+template <typename XT, int T, int CPL, int U, int WARPS, bool K, int SPLIT, bool GRAD, bool BLOCKS>
 __global__ void __launch_bounds__(WARPS * 32) k_estimate(EstArgs a) {
   using CT = typename Store<XT>::CT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -596,31 +591,55 @@ __global__ void __launch_bounds__(WARPS * 32) k_estimate(EstArgs a) {
   const double temp = a.a_from_state ? a.st->a : a.a_host;
   const int32_t *idx = a.u + (int64_t)i * a.m;
   double ell, sig2;
-  if constexpr (USE == kUseAny) {
-    double *blk = a.blk ? a.blk + (int64_t)i * a.G * 2 : nullptr;
-    const RowIO<CT> io;
-    auto eval = [&](auto grad_c, auto blocks_c) {
-      return eval_particle<XT, T, CPL, U, K, decltype(grad_c)::value, decltype(blocks_c)::value, 0,
-                           SPLIT>(W, a, idx, sm, temp, blk, ell, sig2, io, warp, stride);
-    };
-    constexpr std::true_type yes{};
-    constexpr std::false_type no{};
-    if (!(a.grad ? (blk ? eval(yes, yes) : eval(yes, no)) : (blk ? eval(no, yes) : eval(no, no))))
-      return;
-    if (a.grad) {
-      CT *g = reinterpret_cast<CT *>(a.grad) + (int64_t)i * a.p;
-      for (int c = W.lane; c < a.p; c += 32) g[c] = sm.g[c];
-    }
+  double *blk = BLOCKS ? a.blk + (int64_t)i * a.G * 2 : nullptr;
+  if (!eval_particle<XT, T, CPL, U, K, GRAD, BLOCKS, 0, SPLIT>(W, a, idx, sm, temp, blk, ell, sig2,
+                                                               RowIO<CT>(), warp, stride))
+    return;
+  if (GRAD) {
+    CT *g = reinterpret_cast<CT *>(a.grad) + (int64_t)i * a.p;
+    for (int c = W.lane; c < a.p; c += 32) g[c] = sm.g[c];
+  }
+  if (W.lane == 0) {
+    if (a.ell) a.ell[i] = ell;
+    if (a.sig2) a.sig2[i] = sig2;
+    if (!isfinite(ell) || !isfinite(sig2)) set_err(a.st, kErrNonFinite);
+  }
+}
+
+// One warp per particle with all uses in one kernel (chosen by a.grad and a.blk): the gradient of the
+// tiles with eight lanes per row or more, whose schedule alone was slower (p = 101, 16384 particles
+// of m = 5000: 3.53 ms here, 3.87 alone; start of the comparison 3.69).
+template <typename XT, int T, int CPL, int U, int WARPS, bool K>
+__global__ void __launch_bounds__(WARPS * 32) k_estimate_any(EstArgs a) {
+  using CT = typename Store<XT>::CT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * WARPS + warp;
+  if (i >= a.B) return;  // whole warp leaves together; no block-level barriers follow
+  WarpEval<XT, T, CPL, U, K> W;
+  unsigned char *wbase = smem_raw + (size_t)warp * warp_smem_bytes<XT, T, CPL, U>(a.p);
+  W.init(wbase, a.Yo);
+  WarpSmem<CT> sm(reinterpret_cast<CT *>(wbase + WarpEval<XT, T, CPL, U, K>::RING), a.p, T * CPL);
+  const CT *th = reinterpret_cast<const CT *>(a.theta) + (int64_t)i * a.p;
+  for (int c = W.lane; c < a.p; c += 32) sm.th[c] = th[c];
+  __syncwarp();
+  refresh_delta(W, a, sm);
+  const double temp = a.a_from_state ? a.st->a : a.a_host;
+  const int32_t *idx = a.u + (int64_t)i * a.m;
+  double ell, sig2;
+  double *blk = a.blk ? a.blk + (int64_t)i * a.G * 2 : nullptr;
+  if (a.grad) {
+    if (blk)
+      eval_particle<XT, T, CPL, U, K, true, true>(W, a, idx, sm, temp, blk, ell, sig2);
+    else
+      eval_particle<XT, T, CPL, U, K, true, false>(W, a, idx, sm, temp, nullptr, ell, sig2);
+    CT *g = reinterpret_cast<CT *>(a.grad) + (int64_t)i * a.p;
+    for (int c = W.lane; c < a.p; c += 32) g[c] = sm.g[c];
   } else {
-    constexpr bool GRAD = USE == kUseGrad, BLOCKS = USE == kUseCache;
-    double *blk = BLOCKS ? a.blk + (int64_t)i * a.G * 2 : nullptr;
-    if (!eval_particle<XT, T, CPL, U, K, GRAD, BLOCKS, 0, SPLIT>(W, a, idx, sm, temp, blk, ell,
-                                                                 sig2, RowIO<CT>(), warp, stride))
-      return;
-    if (GRAD) {
-      CT *g = reinterpret_cast<CT *>(a.grad) + (int64_t)i * a.p;
-      for (int c = W.lane; c < a.p; c += 32) g[c] = sm.g[c];
-    }
+    if (blk)
+      eval_particle<XT, T, CPL, U, K, false, true>(W, a, idx, sm, temp, blk, ell, sig2);
+    else
+      eval_particle<XT, T, CPL, U, K, false, false>(W, a, idx, sm, temp, nullptr, ell, sig2);
   }
   if (W.lane == 0) {
     if (a.ell) a.ell[i] = ell;
@@ -1001,16 +1020,20 @@ inline int launch_tile(int op, const EstArgs &a, cudaStream_t s) {
     if (e == cudaSuccess) kernel<<<grid, block, smem, s>>>(a);
   };
   if (op == 0) {
-    constexpr int kGrad = T >= 8 ? kUseAny : kUseGrad;
     if (a.grad && a.blk) return (int)cudaErrorInvalidValue;  // (no entry point asks for both)
-    if (split)
-      a.grad  ? go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, kUseGrad>)
-      : a.blk ? go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, kUseCache>)
-              : go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, kUseEst>);
-    else
-      a.grad  ? go(k_estimate<XT, T, CPL, U, WARPS, K, 1, kGrad>)
-      : a.blk ? go(k_estimate<XT, T, CPL, U, WARPS, K, 1, kUseCache>)
-              : go(k_estimate<XT, T, CPL, U, WARPS, K, 1, kUseEst>);
+    if (split) {
+      a.grad  ? go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, true, false>)
+      : a.blk ? go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, false, true>)
+              : go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, false, false>);
+    } else if (a.grad) {
+      if constexpr (T >= 8)
+        go(k_estimate_any<XT, T, CPL, U, WARPS, K>);
+      else
+        go(k_estimate<XT, T, CPL, U, WARPS, K, 1, true, false>);
+    } else {
+      a.blk ? go(k_estimate<XT, T, CPL, U, WARPS, K, 1, false, true>)
+            : go(k_estimate<XT, T, CPL, U, WARPS, K, 1, false, false>);
+    }
   } else if (op == 1) {
     go(k_upm<XT, T, CPL, U, WARPS, K>);
   } else if (op == 2) {
