@@ -265,53 +265,6 @@ __device__ __forceinline__ float rcp_ftz(float x) {
   return y;
 }
 
-// The logistic increment for |D| <= kFarD in FP32 (used above 1/2), from
-//   softplus(eta_bar + D) - softplus(eta_bar) = log((1 - s) + s e^D),
-//   sigma(eta_bar + D) = s e^D / ((1 - s) + s e^D):
-// one exponential, one logarithm and one reciprocal, no case distinction. Root-mean-square error of d
-// against FP64 over eta_bar of sd 1.5: 6e-8 for |D| in [1/2, 1] and 8e-8 in [1, 2] (1.0e-7 and
-// 1.2e-7 for the form row_incr takes beyond kFarD, which has two logarithms); of r 3e-8 and 4e-8 (the
-// same). Above kFarD the logarithm's relative error would count.
-constexpr float kFarD = 2.0f;
-__device__ __forceinline__ void logistic_far(float s, float w, float D, float &d, float &r) {
-  const float se = s * ex2_ftz(D * 1.44269504088896341f);
-  const float den = (1.0f - s) + se;
-  const float wD = w * D;
-  r = (wD + s) - se * rcp_ftz(den);
-  d = fmaf(0.5f * wD, D, fmaf(s, D, -0.693147180559945309f * lg2_ftz(den)));
-}
-
-// The logistic cumulant series of row_incr in FP32: kappa_3 .. kappa_10 as polynomials in w with w (and
-// q for the odd ones) factored out and scaled by 1/(k-1)!, so every constant is the immediate of a
-// scalar FMA; the chain of d divides each by its k.
-__device__ __forceinline__ void logistic_series(float s, float w, float D, float &d, float &r) {
-  const float q = fmaf(s, -2.f, 1.f);
-  const float e4 = (float)(1.0 / 6) - w;
-  const float e6 = fmaf(w, w - 0.25f, (float)(1.0 / 120));
-  const float e8 =
-      fmaf(w, fmaf(w, (float)(1.0 / 3) - w, (float)(-1.0 / 40)), (float)(1.0 / 5040));
-  const float e10 = fmaf(
-      w, fmaf(w, fmaf(w, w - (float)(5.0 / 12), (float)(7.0 / 144)), (float)(-17.0 / 12096)),
-      (float)(1.0 / 362880));
-  const float o3 = 0.5f * q;
-  const float o5 = q * fmaf(w, -0.5f, (float)(1.0 / 24));
-  const float o7 = q * fmaf(w, fmaf(w, 0.5f, (float)(-1.0 / 12)), (float)(1.0 / 720));
-  const float o9 = q * fmaf(w, fmaf(w, fmaf(w, -0.5f, 0.125f), (float)(-1.0 / 160)),
-                            (float)(1.0 / 40320));
-  float2 c = make_float2(0.1f * e10, e10);  // the chains of d and r
-  const float2 DD = make_float2(D, D);
-  c = __ffma2_rn(c, DD, make_float2(o9 * (float)(1.0 / 9), o9));
-  c = __ffma2_rn(c, DD, make_float2(e8 * 0.125f, e8));
-  c = __ffma2_rn(c, DD, make_float2(o7 * (float)(1.0 / 7), o7));
-  c = __ffma2_rn(c, DD, make_float2(e6 * (float)(1.0 / 6), e6));
-  c = __ffma2_rn(c, DD, make_float2(o5 * 0.2f, o5));
-  c = __ffma2_rn(c, DD, make_float2(e4 * 0.25f, e4));
-  c = __ffma2_rn(c, DD, make_float2(o3 * (float)(1.0 / 3), o3));
-  const float nwd2 = -w * (D * D);
-  r = nwd2 * c.y;
-  d = nwd2 * D * c.x;
-}
-
 // Horner steps of the two cumulant-series chains at once (FP32: one packed FMA per step):
 // (pd, pr) = (pd, pr) * D + kappa * (1/k!, 1/(k-1)!).
 template <typename CT>
@@ -328,8 +281,11 @@ __device__ __forceinline__ void horner2<float>(float &pd, float &pr, float D, fl
   pr = v.y;
 }
 
+// short4: the caller has checked |D| <= 1/20 for every lane of the warp (FP32 only); the
+// logistic series then stops at kappa_6 (truncation below 2e-8 of w|D|^3 and w D^2).
 template <int FAM, typename CT>
-__device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT &d, CT &r) {
+__device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT &d, CT &r,
+                                         bool short4 = false) {
   if (FAM == 0) {  // logistic: l = y*eta - log(1 + e^eta); y cancels from d and r
     const CT sb = c.c0, w = c.c1;
     // With K(D) = log(1 - s + s e^D), the cumulant generating function of Bernoulli(s), s = sigma(eta_bar):
@@ -339,6 +295,21 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
     // relative error below 1e-8 in d and 1e-7 in r (1e-15 in FP64). No transcendental, no
     // division, no cancellation.
     constexpr CT kSmall = sizeof(CT) == 8 ? CT(0.05) : CT(0.5);
+    if (sizeof(CT) == 4 && short4) {
+      const CT q = CT(1) - CT(2) * sb;
+      const CT k3 = w * q;
+      const CT k4 = w * (CT(1) - CT(6) * w);
+      const CT k5 = k3 * (CT(1) - CT(12) * w);
+      const CT k6 = w * (CT(1) + w * (CT(-30) + CT(120) * w));
+      CT pd = k6 * CT(1.0 / 720.0), pr = k6 * CT(1.0 / 120.0);
+      horner2(pd, pr, D, k5, 1.0 / 120.0, 1.0 / 24.0);
+      horner2(pd, pr, D, k4, 1.0 / 24.0, 1.0 / 6.0);
+      horner2(pd, pr, D, k3, 1.0 / 6.0, 0.5);
+      const CT D2 = D * D;
+      d = -D2 * D * pd;
+      r = -D2 * pr;
+      return;
+    }
     // FP32: one form per warp (a vote over the lanes evaluating a row here), so a warp whose rows
     // straddle |D| = 1/2 does not run both forms; rows with small |D| in a warp that takes the
     // exp/log form carry that form's absolute error (about 3e-7) instead of the series' relative one
@@ -347,17 +318,7 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
       series = !__any_sync(__activemask(), fabs(D) > kSmall);
     else
       series = fabs(D) <= kSmall;
-    if constexpr (sizeof(CT) == 4) {
-      if (series) {
-        logistic_series(sb, w, D, d, r);
-        return;
-      }
-      if (!__any_sync(__activemask(), fabsf(D) > kFarD)) {
-        logistic_far(sb, w, D, d, r);
-        return;
-      }
-    }
-    if (sizeof(CT) == 8 && series) {
+    if (series) {
       const CT q = CT(1) - CT(2) * sb;
       const CT k3 = w * q;
       const CT k4 = w * (CT(1) - CT(6) * w);
@@ -382,7 +343,7 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
       return;
     }
     if constexpr (sizeof(CT) == 4) {
-      // |D| > kFarD in FP32: with eta = eta_bar + D and softplus(x) = max(x, 0) + log(1 + e^-|x|),
+      // |D| > 1/2 in FP32: with eta = eta_bar + D and softplus(x) = max(x, 0) + log(1 + e^-|x|),
       //   L1 = softplus(eta) - softplus(eta_bar)
       //      = [max(eta, 0) - max(eta_bar, 0)] + log(1 + e^-|eta|) - log(1 + e^-|eta_bar|),
       // where log(1 + e^-|eta_bar|) = -log(max(s, 1 - s)) (1 - s is exact for s >= 1/2), and
@@ -391,12 +352,11 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
       // approximations (MUFU ex2/lg2/rcp) err by about 2e-7 absolute, the size of what d loses
       // to its own cancellation (-L1 + sD + wD^2/2) at this |D| in FP32 anyway.
       const float eb = c.c2, eta = eb + D;
-      const float e = ex2_ftz(-1.44269504088896341f * fabsf(eta)), ope = 1.0f + e;
-      const float ln2 = 0.693147180559945309f;
-      const float lb = ln2 * lg2_ftz(fmaxf(sb, 1.0f - sb));
+      const float e = __expf(-fabsf(eta)), ope = 1.0f + e;
+      const float lb = __logf(fmaxf(sb, 1.0f - sb));
       const float pos = eb >= 0.0f ? (eta >= 0.0f ? D : -eb) : (eta >= 0.0f ? eta : 0.0f);
-      const float L1f = pos + (ln2 * lg2_ftz(ope) + lb);
-      const float inv = rcp_ftz(ope);
+      const float L1f = pos + (__logf(ope) + lb);
+      const float inv = __fdividef(1.0f, ope);
       const float sg = eta >= 0.0f ? inv : e * inv;
       r = fmaf(w, D, sb - sg);
       d = fmaf(0.5f * w * D, D, fmaf(sb, D, -L1f));
