@@ -430,6 +430,21 @@ __device__ __forceinline__ void split_rows(int m, int G, int w, int W, bool bloc
   j1 = min(j1, m);
 }
 
+// One entry of grad (a l_hat - a^2/2 sigma2_hat + log p): bc, cd those of B and C delta, G1 = sum r x,
+// G2 = sum e r x, dbar the mean of e, dth = theta - mu. FP32: every rounding written out, so that
+// the kernels that assemble it agree bit for bit.
+__device__ __forceinline__ float target_grad(float ta, float tnm, float ta2, float bc, float cd,
+                                             float G1, float G2, float dbar, float dth, float iv) {
+  const float like = __fmaf_rn(ta, __fadd_rn(bc, cd), __fmul_rn(tnm, G1));
+  return __fmaf_rn(-dth, iv, __fmaf_rn(-ta2, __fmaf_rn(-dbar, G1, G2), like));
+}
+__device__ __forceinline__ double target_grad(double ta, double tnm, double ta2, double bc, double cd,
+                                              double G1, double G2, double dbar, double dth,
+                                              double iv) {
+  const double pg = -dth * iv;
+  return ta * (bc + cd) + tnm * G1 - ta2 * (G2 - dbar * G1) + pg;
+}
+
 // One evaluation of the estimator for a particle at theta (in sm.th / sm.dl) by one warp, or, with
 // SPLIT > 1, by the SPLIT warps of its CTA (warp `part` this one; each has its own sm, `stride` bytes
 // apart): every warp sums its own rows, and warp 0 merges them. Returns whether this warp is the one
@@ -523,8 +538,8 @@ __device__ __forceinline__ bool eval_particle(const WarpEval<XT, T, CPL, U, K> &
     qlin += (double)(dc * (bc + CT(0.5) * cd));
     if (GRAD) {
       const CT G1 = sm.G1[c], G2 = sm.G2[c];
-      const CT pg = -(sm.th[c] - ldg_ct<CT>(a.mu_ct, c)) * ldg_ct<CT>(a.ivar_ct, c);
-      sm.g[c] = ta * (bc + cd) + tnm * G1 - ta2 * (G2 - cdbar * G1) + pg;
+      sm.g[c] = target_grad(ta, tnm, ta2, bc, cd, G1, G2, cdbar, sm.th[c] - ldg_ct<CT>(a.mu_ct, c),
+                            ldg_ct<CT>(a.ivar_ct, c));
     }
   }
   qlin = warp_sum(qlin);

@@ -130,8 +130,8 @@ constexpr int kTwoWarpRows = 512;
 // Warps per CTA of the default resident tile for p covariates and m subsample rows (measured on
 // GB300, 1024 particles per problem): one warp while a warp's rows outweigh the per-pass work
 // that every warp repeats (p 9..24 up to m = 400, p > 24 up to m = 160; at p <= 8 two warps
-// always do better), two up to m = 512, else four. Above 40 covariates four (us per trajectory of
-// L = 20 at p = 50: 229 against 241 with eight at m = 1250, 100 against 176 at m = 512).
+// always do better), two up to m = 512, else four. Above 40 covariates the tiles' own count
+// (resident_wide.cuh), listed as four.
 inline int res_default_warps(int p, int m) {
   if (p > 40) return 4;
   if (p > 8 && m <= (p <= 24 ? 400 : 160)) return 1;

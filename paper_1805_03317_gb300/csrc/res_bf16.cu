@@ -10,7 +10,7 @@ using XT = __nv_bfloat16;
 // tiles hold two columns per lane. Tiles 10..16 are the two-warp CTAs (res_bf16_w2.cu) and 17..23
 // the one-warp CTAs (res_bf16_w1.cu) for small subsamples, where the per-pass work that every
 // warp repeats outweighs the rows. Tiles 24 and 25 (res_bf16_wide.cu) take rows of 41 to 64
-// covariates on the warp-level tensor-core path (resident_mma.cuh).
+// covariates in the streamed kernel's arithmetic (resident_wide.cuh).
 const Tile kResTiles[] = {{1, 8, 1, 4},  {1, 16, 1, 4}, {1, 24, 1, 4}, {1, 32, 1, 4}, {1, 16, 1, 8},
                           {1, 24, 1, 8}, {1, 20, 1, 4}, {1, 12, 1, 4}, {0, 32, 1, 8}, {1, 40, 1, 4},
                           {1, 8, 1, 2},  {1, 12, 1, 2}, {1, 16, 1, 2}, {1, 20, 1, 2}, {1, 24, 1, 2},
