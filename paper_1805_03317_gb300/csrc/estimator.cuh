@@ -135,8 +135,8 @@ struct WarpEval {
 
   // One pass over rows idx[0..nrows). GRAD: accumulates the gradient partials sum r x, sum d r x
   // over this lane's slots into g1, g2. Returns S = sum d and Q = sum d^2 on every lane; BLOCKS
-  // also writes per-block (sum d, sum d^2) to blk_out[2G]: the rows are whole blocks, from block
-  // g_first on, of the floor partition of mtot rows into G blocks.
+  // also writes per-block (sum d, sum d^2) of the floor partition of the nrows rows into G blocks
+  // to blk_out[2G].
   // The sums are of e = d - K (returned in Ksh, warp-uniform: the d of row 0), so
   // Ssum = sum e and Qsum = sum e^2; g2 accumulates e r x. BLOCKS writes the unshifted FP64 block
   // sums (sum d, sum d^2) rebuilt from the shifted ones.
@@ -145,8 +145,7 @@ struct WarpEval {
                                        const int32_t *idx, int nrows, int fam, CT inv_s2, CT *g1,
                                        CT *g2, double *blk_out, int G, double &Ssum, double &Qsum,
                                        double &Ksh, DevState *st,
-                                       const RowIO<CT> &io = RowIO<CT>(), int cv1 = 0,
-                                       int g_first = 0, int mtot = 0) const {
+                                       const RowIO<CT> &io = RowIO<CT>(), int cv1 = 0) const {
     const int nsw = (nrows + 31) >> 5;
     // rows past the end copy the last row again (already on chip) and are masked out
     const int klast = nrows > 0 ? idx[nrows - 1] : 0;
@@ -194,35 +193,19 @@ struct WarpEval {
       }
       cp_async_commit();  // one group per sweep (empty past the end) keeps the counting uniform
     };
-    CT sd = CT(0), sd2 = CT(0);  // lane sums of e, e^2 (BLOCKS: of the open block since its last flush)
+    CT sd = CT(0), sd2 = CT(0);  // lane sums of e, e^2 (BLOCKS: of one sweep and block)
     CT K = CT(0);               // shift of the sums: d of row 0 (set at sweep 0)
     Ssum = Qsum = 0.0;
-    // BLOCKS: the open block cg, local rows up to jend, and what its flushes have summed
-    int cg = g_first, nfl = 0;
-    const int j0g = BLOCKS ? block_first(g_first, mtot, G) : 0;
-    int jend = BLOCKS ? block_first(cg + 1, mtot, G) - j0g : 0;
+    // BLOCKS: the open block cg, its rows up to jend, its sums so far
+    int cg = 0, jend = BLOCKS ? block_first(1, nrows, G) : 0;
     double cs = 0.0, cq = 0.0;
-    constexpr bool EACH = sizeof(CT) == 8;  // FP64 rows: a sum per sweep (their terms dominate)
-    auto flush = [&]() {
+    auto flush = [&]() {  // the lane sums of one sweep's rows of the open block
       const CT bs = warp_sum(sd), bq = warp_sum(sd2);
-      if (EACH) {
-        Ssum += (double)bs;
-        Qsum += (double)bq;
-      }
-      cs = nfl ? cs + (double)bs : (double)bs;
-      cq = nfl ? cq + (double)bq : (double)bq;
-      ++nfl;
+      cs += (double)bs;
+      cq += (double)bq;
+      Ssum += (double)bs;
+      Qsum += (double)bq;
       sd = sd2 = CT(0);
-    };
-    auto close_block = [&]() {
-      flush();
-      if (lane == 0) {
-        blk_out[2 * cg] = cs;
-        blk_out[2 * cg + 1] = cq;
-      }
-      nfl = 0;
-      ++cg;
-      jend = block_first(cg + 1, mtot, G) - j0g;
     };
     // partial x'delta of the group's T rows over this lane's slots, reduce-scattered: the full D of
     // the row this lane owns
@@ -276,23 +259,33 @@ struct WarpEval {
       if (s == 0) K = __shfl_sync(0xffffffffu, d, 0);  // every lane is here at sweep 0
       d = valid ? d - K : CT(0);  // from here on d holds e = d - K
       if (BLOCKS) {
-        // Lane sums within a block, flushed through a warp tree into FP64 when the block closes (or
-        // after 8 sweeps): an FP64 add holds the warp's pipe for 64 cycles, so not one per sweep
-        // (1000 rows, 10 blocks: 123 us for 4096 particles with sums per sweep, 84 us now).
+        // a sweep's rows of a block through a warp tree, the trees' results in FP64 (lane sums over
+        // eight sweeps would save a third of the refresh, 84 instead of 123 us for 4096 particles of
+        // 1000 rows, but with FP32 sums of 256 rows)
         int rest = 0;  // rows of the sweep before this one belong to closed blocks
-        while (jend <= min((s << 5) + 32, nrows)) {  // (no block is empty: G <= m)
+        const int send = min((s << 5) + 32, nrows);
+        while (jend <= send) {  // (no block is empty: G <= m)
           if (j >= rest && j < jend) {
-            sd += d;
-            sd2 = fma(d, d, sd2);
+            sd = d;
+            sd2 = d * d;
           }
+          flush();
           rest = jend;
-          close_block();
+          if (lane == 0) {  // the block's unshifted FP64 sums from the shifted ones
+            const double ng = (double)(jend - block_first(cg, nrows, G)), k = (double)K;
+            blk_out[2 * cg] = fma(ng, k, cs);
+            blk_out[2 * cg + 1] = cq + k * fma(ng, k, 2.0 * cs);
+          }
+          cs = cq = 0.0;
+          jend = block_first(++cg + 1, nrows, G);
         }
-        if (j >= rest && j < nrows) {
-          sd += d;
-          sd2 = fma(d, d, sd2);
+        if (rest < send) {
+          if (j >= rest && j < send) {
+            sd = d;
+            sd2 = d * d;
+          }
+          flush();
         }
-        if (EACH ? jend > min((s << 5) + 32, nrows) && rest < nrows : (s & 7) == 7) flush();
       } else {
         sd += d;
         sd2 = fma(d, d, sd2);
@@ -363,24 +356,7 @@ struct WarpEval {
     }
     cp_async_wait<0>();
     Ksh = (double)K;
-    if (BLOCKS) {
-      // totals, and the blocks' unshifted FP64 sums from the shifted ones, one block per lane
-      __syncwarp();
-      for (int g = g_first + lane; g < cg; g += 32) {
-        const double ng = (double)(block_first(g + 1, mtot, G) - block_first(g, mtot, G));
-        const double se = blk_out[2 * g], qe = blk_out[2 * g + 1];
-        if (!EACH) {
-          Ssum += se;
-          Qsum += qe;
-        }
-        blk_out[2 * g] = fma(ng, Ksh, se);
-        blk_out[2 * g + 1] = qe + Ksh * fma(ng, Ksh, 2.0 * se);
-      }
-      if (!EACH) {
-        Ssum = warp_sum(Ssum);
-        Qsum = warp_sum(Qsum);
-      }
-    } else {
+    if (!BLOCKS) {
       Ssum = warp_sum((double)sd);
       Qsum = warp_sum((double)sd2);
     }
@@ -416,18 +392,13 @@ template <typename CT> __device__ __forceinline__ CT ldg_ct(const void *p, int i
   return __ldg(reinterpret_cast<const CT *>(p) + i);
 }
 
-// The rows of a particle that warp w of a CTA takes when the CTA's W warps share one particle: whole
-// sweeps, or whole blocks where the block sums are wanted. j0, j1: the rows; g0: their first block.
-__device__ __forceinline__ void split_rows(int m, int G, int w, int W, bool blocks, int &j0, int &j1,
-                                           int &g0) {
-  // parts rounded up, so that the first warp is never without rows (its shift is the merge's)
-  const int n = blocks ? G : (m + 31) >> 5;
-  const int p0 = (int)(((int64_t)w * n + W - 1) / W), p1 = (int)(((int64_t)(w + 1) * n + W - 1) / W);
-  g0 = blocks ? p0 : 0;
-  j0 = blocks ? block_first(p0, m, G) : 32 * p0;
-  j1 = blocks ? block_first(p1, m, G) : 32 * p1;
-  j0 = min(j0, m);
-  j1 = min(j1, m);
+// The rows [j0, j1) of a particle that warp w of a CTA takes when the CTA's W warps share one
+// particle: whole sweeps, the parts rounded up, so that the first warp is never without rows (its
+// shift is the merge's).
+__device__ __forceinline__ void split_rows(int m, int w, int W, int &j0, int &j1) {
+  const int n = (m + 31) >> 5;
+  j0 = min(32 * (int)(((int64_t)w * n + W - 1) / W), m);
+  j1 = min(32 * (int)(((int64_t)(w + 1) * n + W - 1) / W), m);
 }
 
 // One entry of grad (a l_hat - a^2/2 sigma2_hat + log p): bc, cd those of B and C delta, G1 = sum r x,
@@ -466,17 +437,18 @@ __device__ __forceinline__ bool eval_particle(const WarpEval<XT, T, CPL, U, K> &
 #pragma unroll
   for (int s = 0; s < CPL; ++s) g1[s] = g2[s] = CT(0);
   double S, Q, Ks;  // sums of e = d - Ks and e^2, and the shift Ks
-  int j0 = 0, j1 = a.m, gb0 = 0;
+  int j0 = 0, j1 = a.m;
   RowIO<CT> io = io_;
+  static_assert(SPLIT == 1 || !BLOCKS, "block sums have one order");
   if constexpr (SPLIT > 1) {
-    split_rows(a.m, a.G, part, SPLIT, BLOCKS, j0, j1, gb0);
+    split_rows(a.m, part, SPLIT, j0, j1);
     if (MODE == 1) {
       io.dsave += j0;
       io.rsave += j0;
     }
   }
   W.template rows<GRAD, BLOCKS, MODE>(Xp, a.S, a.n, idx + j0, j1 - j0, a.fam, inv_s2, g1, g2,
-                                      blk_out, a.G, S, Q, Ks, a.st, io, a.cv_order == 1, gb0, a.m);
+                                      blk_out, a.G, S, Q, Ks, a.st, io, a.cv_order == 1);
   const double nm = (double)a.n / (double)a.m;
   if (GRAD) {
     // reduce the gradient partials over the row slots of the warp
@@ -733,9 +705,9 @@ __global__ void __launch_bounds__(WARPS * 32) k_backward(EstArgs a) {
 #pragma unroll
   for (int e = 0; e < CPL; ++e) g1[e] = g2[e] = CT(0);
   double S_, Q_, K_;
-  int j0 = 0, j1 = m, gb0 = 0;
+  int j0 = 0, j1 = m;
   if constexpr (SPLIT > 1) {
-    split_rows(m, a.G, warp, WARPS, false, j0, j1, gb0);
+    split_rows(m, warp, WARPS, j0, j1);
     io.dsaved += j0;
     io.rsaved += j0;
   }
@@ -1027,9 +999,9 @@ template <typename XT, int T, int CPL, int U, int WARPS, bool K = false>
 inline int launch_tile(int op, const EstArgs &a, cudaStream_t s) {
   const size_t smem = (size_t)WARPS * warp_smem_bytes<XT, T, CPL, U>(a.p);
   if (a.B <= 0) return 0;
-  // (the cache of FP64 states keeps one summation order for every N)
+  // (the cache keeps one summation order for every N: the moves start from it)
   const bool split = WARPS > 1 && (op == 0 || op >= 3) && a.B <= kSplitParticles<typename Store<XT>::CT> &&
-                     !(sizeof(XT) == 8 && a.blk);
+                     !a.blk;
   const dim3 grid(split ? a.B : (a.B + WARPS - 1) / WARPS), block(WARPS * 32);
   cudaError_t e = cudaSuccess;
   auto go = [&](auto *kernel) {
@@ -1039,9 +1011,8 @@ inline int launch_tile(int op, const EstArgs &a, cudaStream_t s) {
   if (op == 0) {
     if (a.grad && a.blk) return (int)cudaErrorInvalidValue;  // (no entry point asks for both)
     if (split) {
-      a.grad  ? go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, true, false>)
-      : a.blk ? go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, false, true>)
-              : go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, false, false>);
+      a.grad ? go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, true, false>)
+             : go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, false, false>);
     } else if (a.grad) {
       if constexpr (T >= 8)
         go(k_estimate_any<XT, T, CPL, U, WARPS, K>);

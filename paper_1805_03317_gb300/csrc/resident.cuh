@@ -351,13 +351,13 @@ __device__ __forceinline__ void res_particle(const EstArgs &a, int i, bool reloa
   }
   set_delta();
   // shift of the row sums (identical in every warp): the cached subsample mean of d at this
-  // particle's current theta and u (any value near the mean serves)
+  // particle's current theta and u, in FP64: its last bit is one of e's
   CT Ksh = CT(0);
   if (a.blk) {
     const double *bc = a.blk + (int64_t)i * G * 2;
-    CT s0 = CT(0);
-    for (int g = lane; g < G; g += 32) s0 += (CT)bc[2 * g];
-    Ksh = warp_sum(s0) * (CT)inv_m;
+    double s0 = 0.0;
+    for (int g = lane; g < G; g += 32) s0 += bc[2 * g];
+    Ksh = (CT)(warp_sum(s0) * inv_m);
     if (!isfinite(Ksh)) Ksh = CT(0);
   }
   cp_async_wait_all();

@@ -26,6 +26,14 @@ GRADS = {
 }
 MOVES = {
     "move_logistic_bf16_p3": ("logistic", "bf16", (6000, 3, 256, 58, 4, 17), 1.0, 0.05, 0.03),
+    "move_student_t_bf16_p50": ("student_t", "bf16", (6000, 50, 192, 200, 8, 6), 3.0, 0.03, 0.1),
+    "move_student_t_bf16_p60": ("student_t", "bf16", (6000, 60, 192, 90, 8, 6), 3.0, 0.03, 0.1),
+    "move_student_t_bf16_p101": ("student_t", "bf16", (6000, 101, 128, 200, 8, 4), 3.0, 0.03, 0.1),
+    "move_student_t_bf16_p12": ("student_t", "bf16", (6000, 12, 256, 300, 11, 10), 3.0, 0.03, 0.1),
+    "move_logistic_bf16_p20": ("logistic", "bf16", (6000, 20, 256, 300, 7, 10), 0.5, 0.05, 0.03),
+    "move_logistic_f32_p13": ("logistic", "f32", (6000, 13, 256, 130, 7, 10), 0.5, 0.05, 0.03),
+    "move_probit_f32_p13": ("probit", "f32", (6000, 13, 256, 130, 7, 10), 0.5, 0.05, 0.03),
+    "move_poisson_bf16_p8": ("poisson", "bf16", (6000, 8, 256, 130, 7, 10), 0.5, 0.05, 0.03),
 }
 
 
