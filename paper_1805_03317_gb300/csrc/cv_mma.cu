@@ -9,9 +9,11 @@
 // MMA's canonical no-swizzle MN-major layout (16-byte cp.async units), one thread per row forms
 // eta = x'theta and the family terms in FP64 (A, and l' for B), the same thread writes its row of
 // the three B-operand tiles, one thread issues 3 x 8 MMAs (K = 16 each) and commits them to an
-// mbarrier. Every kDrain tiles the FP32 accumulator is read back (tcgen05.ld) and added to FP64
+// mbarrier. After kDrain tiles the FP32 accumulator is read back (tcgen05.ld) and added to FP64
 // accumulators of the upper triangle in shared memory; B is accumulated in FP64 by column
-// threads. Per-CTA partials use the layout of the SIMT moment kernel, so the same FP64 reduction
+// threads. Which tiles share an FP32 accumulation depends on n alone, not on how many CTAs run: with
+// one chain of tiles per SM (tile mod chains), kDrain successive tiles of a chain are one work item
+// and CTAs take items. C's last FP32 bit decides last bits of every gradient. Per-CTA partials use the layout of the SIMT moment kernel, so the same FP64 reduction
 // (fixed order over blocks) finishes A, B and C.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -134,7 +136,7 @@ template <int FAM>
 __global__ void __launch_bounds__(kRows) k_cv_mma(const __nv_bfloat16 *Xp, int64_t n, int p, int S,
                                                   int Yo, double s2, double nu,
                                                   const double *theta, double *part, int N,
-                                                  int ncols) {
+                                                  int ncols, int chains) {
   extern __shared__ __align__(128) unsigned char sm[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nvx = (p + 7) / 8;   // 16-byte units of covariates per row
@@ -178,8 +180,18 @@ __global__ void __launch_bounds__(kRows) k_cv_mma(const __nv_bfloat16 *Xp, int64
   int since_drain = 0;
   bool timed_out = false;
   const int64_t ntiles = (n + kRows - 1) / kRows;
-  for (int64_t tile = blockIdx.x; tile < ntiles && !timed_out; tile += gridDim.x) {
+  // work item (q, b): tiles b + chains (4 q + 0 .. 3), one FP32 accumulation
+  const int64_t step = (int64_t)kDrain * chains, nitems = (ntiles + step - 1) / step * chains;
+  int64_t item = blockIdx.x;
+  auto first_tile = [&](int64_t w) { return w / chains * step + w % chains; };
+  int64_t tile = first_tile(item);
+  while (item < nitems && !timed_out) {
     const int64_t r0 = tile * kRows;
+    if (r0 >= n) {  // (the last items of a chain may be short or empty)
+      item += gridDim.x;
+      tile = first_tile(item);
+      continue;
+    }
     // 1. the tile's covariates, MN-major (a unit = 8 consecutive columns of one row)
     for (int u = tid; u < kRows * nvx; u += kRows) {
       const int k = u / nvx, c = u - k * nvx;
@@ -274,9 +286,9 @@ __global__ void __launch_bounds__(kRows) k_cv_mma(const __nv_bfloat16 *Xp, int64
     phase ^= 1u;
     tc_fence_after();
     ++since_drain;
-    const bool last = tile + gridDim.x >= ntiles;
+    const bool last = since_drain == kDrain || tile + chains >= ntiles;
     // 5. drain the FP32 accumulator into the FP64 upper triangle
-    if (!timed_out && (since_drain == kDrain || last)) {
+    if (!timed_out && last) {
       const int i = warp * 32 + lane;  // TMEM lane = covariate index i
       for (int j0 = 0; j0 < N; j0 += 8) {
         float v[8];
@@ -291,6 +303,12 @@ __global__ void __launch_bounds__(kRows) k_cv_mma(const __nv_bfloat16 *Xp, int64
         }
       }
       since_drain = 0;
+    }
+    if (last) {
+      item += gridDim.x;
+      tile = first_tile(item);
+    } else {
+      tile += chains;
     }
     tc_fence_before();
     __syncthreads();  // the tile's shared memory and the accumulator may be reused
@@ -359,12 +377,14 @@ int launch_fam(const __nv_bfloat16 *Xp, int64_t n, int p, int S, int Yo, double 
   if (per_sm * cols > 512) per_sm = 512 / cols;  // every resident CTA gets its columns at once
   if (per_sm < 1) per_sm = 1;
   const int64_t ntiles = (n + kRows - 1) / kRows;
+  const int chains = ntiles < sms ? (int)ntiles : sms;
+  const int64_t nitems = (ntiles + kDrain * chains - 1) / (kDrain * chains) * chains;
   int64_t grid = (int64_t)per_sm * sms;
   if (grid > maxblocks) grid = maxblocks;
-  if (grid > ntiles) grid = ntiles;
-  if (grid < 1) grid = 1;
+  if (grid > nitems) grid = nitems;
   *nblocks = (int)grid;
-  k_cv_mma<FAM><<<(int)grid, kRows, smem, s>>>(Xp, n, p, S, Yo, s2, nu, theta, part, N, cols);
+  k_cv_mma<FAM><<<(int)grid, kRows, smem, s>>>(Xp, n, p, S, Yo, s2, nu, theta, part, N, cols,
+                                             chains);
   return (int)cudaGetLastError();
 }
 

@@ -30,6 +30,10 @@ MOVES = {
     "move_student_t_bf16_p60": ("student_t", "bf16", (6000, 60, 192, 90, 8, 6), 3.0, 0.03, 0.1),
     "move_student_t_bf16_p101": ("student_t", "bf16", (6000, 101, 128, 200, 8, 4), 3.0, 0.03, 0.1),
     "move_student_t_bf16_p12": ("student_t", "bf16", (6000, 12, 256, 300, 11, 10), 3.0, 0.03, 0.1),
+    "move_student_t_bf16_p12_n60000": (
+        "student_t", "bf16", (60000, 12, 256, 300, 11, 10), 3.0, 0.01, 0.02),
+    "move_student_t_bf16_p50_n120000": (
+        "student_t", "bf16", (120000, 50, 128, 300, 11, 6), 3.0, 0.01, 0.02),
     "move_logistic_bf16_p20": ("logistic", "bf16", (6000, 20, 256, 300, 7, 10), 0.5, 0.05, 0.03),
     "move_logistic_f32_p13": ("logistic", "f32", (6000, 13, 256, 130, 7, 10), 0.5, 0.05, 0.03),
     "move_probit_f32_p13": ("probit", "f32", (6000, 13, 256, 130, 7, 10), 0.5, 0.05, 0.03),
