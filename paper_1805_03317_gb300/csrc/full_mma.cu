@@ -359,26 +359,20 @@ __global__ void __launch_bounds__(kThreads) k_full_mma(
         const float *yt = ys + b * kR;
         const bool fast = full_p && t0 + kR <= r1;
         const int c_lo = half * 64;
-        uint32_t v[2][16];
-        ld16_issue(tE + tlane + (uint32_t)c_lo, v[0]);
-#pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          const int c0 = c_lo + 16 * ch;
-          float d[16];
+        // the 16 columns from c0: their sum of l into the particle's, l' as two BF16 terms into P
+        auto chunk = [&](int c0, const uint32_t (&v)[16]) {
+          float d[16], ls;
           const float4 y4[4] = {*reinterpret_cast<const float4 *>(yt + c0),
                                 *reinterpret_cast<const float4 *>(yt + c0 + 4),
                                 *reinterpret_cast<const float4 *>(yt + c0 + 8),
                                 *reinterpret_cast<const float4 *>(yt + c0 + 12)};
           const float *yy = reinterpret_cast<const float *>(y4);
-          ld16_wait(v[ch & 1]);
-          if (ch < 3) ld16_issue(tE + tlane + (uint32_t)(c0 + 16), v[(ch + 1) & 1]);
-          float ls;
-          if (fast) {
-            ls = fam_chunk<FAM, false>(v[ch & 1], yy, inv_s2, nu, 0u, d);
+          if (FAM != 1 && fast) {
+            ls = fam_chunk<FAM, false>(v, yy, inv_s2, nu, 0u, d);
           } else {
             const int64_t left = r1 - (t0 + c0);
             const uint32_t ok = !live || left <= 0 ? 0u : left >= 16 ? 0xFFFFu : (1u << left) - 1u;
-            ls = fam_chunk<FAM, true>(v[ch & 1], yy, inv_s2, nu, ok, d);
+            ls = fam_chunk<FAM, true>(v, yy, inv_s2, nu, ok, d);
           }
           lsum += (double)ls;
           uint4 hi0, lo0, hi1, lo1;
@@ -389,6 +383,31 @@ __global__ void __launch_bounds__(kThreads) k_full_mma(
           *reinterpret_cast<uint4 *>(Pt + uoff(pr, q0 + 1)) = hi1;
           *reinterpret_cast<uint4 *>(Pt + 16 * kStrip + uoff(pr, q0)) = lo0;
           *reinterpret_cast<uint4 *>(Pt + 16 * kStrip + uoff(pr, q0 + 1)) = lo1;
+        };
+        if constexpr (FAM != 1 && FAM != 4) {
+          // few instructions per column: the four chunks unrolled, the next one's load in flight
+          uint32_t v[2][16];
+          ld16_issue(tE + tlane + (uint32_t)c_lo, v[0]);
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch) {
+            const int c0 = c_lo + 16 * ch;
+            ld16_wait(v[ch & 1]);
+            if (ch < 3) ld16_issue(tE + tlane + (uint32_t)(c0 + 16), v[(ch + 1) & 1]);
+            chunk(c0, v[ch & 1]);
+          }
+        } else {
+          // log1p and a division (Student-t), erfc and erfcx (probit) per column: four chunks with and
+          // without masks no longer fit the instruction caches, and of probit's terms one copy is
+          // enough. us for 612 particles over 400 000 rows of 24, unrolled / with and without masks /
+          // one copy: probit 2504 / 1923 / 1632, Student-t 806 / 696 / 767; unrolled against one copy:
+          // Poisson 251 / 438, Gaussian 262 / 383.
+#pragma unroll 1
+          for (int c0 = c_lo; c0 < c_lo + 64; c0 += 16) {
+            uint32_t v[16];
+            ld16_issue(tE + tlane + (uint32_t)c0, v);
+            ld16_wait(v);
+            chunk(c0, v);
+          }
         }
       }
       asm volatile("cp.async.wait_all;\n" ::: "memory");  // the next tile has landed
