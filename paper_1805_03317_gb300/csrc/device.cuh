@@ -190,11 +190,7 @@ template <typename CT, int K0> __device__ __forceinline__ CT exp_tail(CT D) {
 }
 
 // log Phi(z) and lambda(z) = phi(z)/Phi(z) from CUDA's erfc/erfcx.
-// A translation unit may have it called instead of inlined (defined before this header is included).
-#ifndef SUBSMC_LOG_PHI_CALL
-#define SUBSMC_LOG_PHI_CALL __forceinline__
-#endif
-template <typename CT> __device__ SUBSMC_LOG_PHI_CALL void log_phi_(CT z, CT &lp, CT &lam) {
+template <typename CT> __device__ __forceinline__ void log_phi_(CT z, CT &lp, CT &lam) {
   const CT x = -z * CT(0.70710678118654752440);
   const CT ex = erfcx(x);
   lam = CT(0.79788456080286535588) / ex;

@@ -1,8 +1,4 @@
 // Estimator kernels for bf16 storage of X: one instantiation per compiled tile shape.
-// log_phi_ stays a call here: inlined, the probit terms crowd the sweep loop that all families share
-// (Poisson p = 50, 8192 particles of m = 2000: 400 us inlined, 394 as a call; GAM p = 101, 16384 of
-// m = 5000: 3.68 ms, 3.53).
-#define SUBSMC_LOG_PHI_CALL __noinline__
 #include "estimator.cuh"
 
 namespace subsmc {

@@ -65,12 +65,6 @@ template <typename CT> struct RowIO {
 // barrier. (When the tiles' chunks end before the tail, the owner copies its tail itself.)
 // Chunk vectors are XOR-swizzled so that 128-bit reads of 8 consecutive lanes hit distinct bank
 // groups; chunk vectors that lie past the covariates are never copied and stay zero.
-// First row of block g of the floor partition of m rows into G blocks (g <= G <= m < 2^31).
-__device__ __forceinline__ int block_first(int g, int m, int G) {
-  const uint64_t v = (uint64_t)(uint32_t)g * (uint32_t)m;
-  return (v >> 32) ? (int)(v / (uint32_t)G) : (int)((uint32_t)v / (uint32_t)G);
-}
-
 template <typename XT, int T, int CPL, int NST, bool PIPE = false>
 struct WarpEval {
   using SD = Store<XT>;
@@ -193,19 +187,22 @@ struct WarpEval {
       }
       cp_async_commit();  // one group per sweep (empty past the end) keeps the counting uniform
     };
-    CT sd = CT(0), sd2 = CT(0);  // lane sums of e, e^2 (BLOCKS: of one sweep and block)
+    if (BLOCKS) {
+      for (int h = lane; h < 2 * G; h += 32) blk_out[h] = 0.0;  // blocks with no rows stay zero
+      __syncwarp();
+    }
+    CT sd = CT(0), sd2 = CT(0);
+    double cs = 0.0, cq = 0.0;  // BLOCKS: shifted sums of the open block cg
+    int cg = -1;
     CT K = CT(0);               // shift of the sums: d of row 0 (set at sweep 0)
     Ssum = Qsum = 0.0;
-    // BLOCKS: the open block cg, its rows up to jend, its sums so far
-    int cg = 0, jend = BLOCKS ? block_first(1, nrows, G) : 0;
-    double cs = 0.0, cq = 0.0;
-    auto flush = [&]() {  // the lane sums of one sweep's rows of the open block
-      const CT bs = warp_sum(sd), bq = warp_sum(sd2);
-      cs += (double)bs;
-      cq += (double)bq;
-      Ssum += (double)bs;
-      Qsum += (double)bq;
-      sd = sd2 = CT(0);
+    // close block g: its unshifted FP64 sums from the shifted ones
+    auto close_block = [&](int g) {
+      const double ng = (double)((int)(((int64_t)(g + 1) * nrows) / G) -
+                                 (int)(((int64_t)g * nrows) / G));
+      const double k = (double)K;
+      blk_out[2 * g] = fma(ng, k, cs);
+      blk_out[2 * g + 1] = cq + k * fma(ng, k, 2.0 * cs);
     };
     // partial x'delta of the group's T rows over this lane's slots, reduce-scattered: the full D of
     // the row this lane owns
@@ -258,33 +255,24 @@ struct WarpEval {
       }
       if (s == 0) K = __shfl_sync(0xffffffffu, d, 0);  // every lane is here at sweep 0
       d = valid ? d - K : CT(0);  // from here on d holds e = d - K
-      if (BLOCKS) {
-        // a sweep's rows of a block through a warp tree, the trees' results in FP64 (lane sums over
-        // eight sweeps would save a third of the refresh, 84 instead of 123 us for 4096 particles of
-        // 1000 rows, but with FP32 sums of 256 rows)
-        int rest = 0;  // rows of the sweep before this one belong to closed blocks
-        const int send = min((s << 5) + 32, nrows);
-        while (jend <= send) {  // (no block is empty: G <= m)
-          if (j >= rest && j < jend) {
-            sd = d;
-            sd2 = d * d;
+      if (BLOCKS) {  // block of row j: largest g with floor(g nrows / G) <= j
+        const int r1 = min((s << 5) + 31, nrows - 1);
+        const int gA = (int)(((unsigned)((s << 5) + 1) * (unsigned)G - 1u) / (unsigned)nrows);
+        const int gB = (int)(((unsigned)(r1 + 1) * (unsigned)G - 1u) / (unsigned)nrows);
+        const int gj =
+            j < nrows ? (int)(((unsigned)(j + 1) * (unsigned)G - 1u) / (unsigned)nrows) : -1;
+        for (int g = gA; g <= gB; ++g) {
+          const CT bs = warp_sum(gj == g ? d : CT(0));
+          const CT bq = warp_sum(gj == g ? d * d : CT(0));
+          if (g != cg) {
+            if (cg >= 0 && lane == 0) close_block(cg);
+            cg = g;
+            cs = cq = 0.0;
           }
-          flush();
-          rest = jend;
-          if (lane == 0) {  // the block's unshifted FP64 sums from the shifted ones
-            const double ng = (double)(jend - block_first(cg, nrows, G)), k = (double)K;
-            blk_out[2 * cg] = fma(ng, k, cs);
-            blk_out[2 * cg + 1] = cq + k * fma(ng, k, 2.0 * cs);
-          }
-          cs = cq = 0.0;
-          jend = block_first(++cg + 1, nrows, G);
-        }
-        if (rest < send) {
-          if (j >= rest && j < send) {
-            sd = d;
-            sd2 = d * d;
-          }
-          flush();
+          cs += (double)bs;
+          cq += (double)bq;
+          Ssum += (double)bs;
+          Qsum += (double)bq;
         }
       } else {
         sd += d;
@@ -355,14 +343,15 @@ struct WarpEval {
       }
     }
     cp_async_wait<0>();
-    Ksh = (double)K;
-    if (!BLOCKS) {
+    if (BLOCKS) {
+      if (cg >= 0 && lane == 0) close_block(cg);
+    } else {
       Ssum = warp_sum((double)sd);
       Qsum = warp_sum((double)sd2);
     }
+    Ksh = (double)K;
   }
 };
-
 
 // Shared-memory scratch of one warp: theta, delta, rho, grad, v [p each] and the reduced gradient
 // partials G1, G2 [T*CPL each], all in the state type.
@@ -392,15 +381,6 @@ template <typename CT> __device__ __forceinline__ CT ldg_ct(const void *p, int i
   return __ldg(reinterpret_cast<const CT *>(p) + i);
 }
 
-// The rows [j0, j1) of a particle that warp w of a CTA takes when the CTA's W warps share one
-// particle: whole sweeps, the parts rounded up, so that the first warp is never without rows (its
-// shift is the merge's).
-__device__ __forceinline__ void split_rows(int m, int w, int W, int &j0, int &j1) {
-  const int n = (m + 31) >> 5;
-  j0 = min(32 * (int)(((int64_t)w * n + W - 1) / W), m);
-  j1 = min(32 * (int)(((int64_t)(w + 1) * n + W - 1) / W), m);
-}
-
 // One entry of grad (a l_hat - a^2/2 sigma2_hat + log p): bc, cd those of B and C delta, G1 = sum r x,
 // G2 = sum e r x, dbar the mean of e, dth = theta - mu. FP32: every rounding written out, so that
 // the kernels that assemble it agree bit for bit.
@@ -416,20 +396,61 @@ __device__ __forceinline__ double target_grad(double ta, double tnm, double ta2,
   return ta * (bc + cd) + tnm * G1 - ta2 * (G2 - dbar * G1) + pg;
 }
 
-// One evaluation of the estimator for a particle at theta (in sm.th / sm.dl) by one warp, or, with
-// SPLIT > 1, by the SPLIT warps of its CTA (warp `part` this one; each has its own sm, `stride` bytes
-// apart): every warp sums its own rows, and warp 0 merges them. Returns whether this warp is the one
-// that holds the result. Reads rows of idx[0..m); GRAD: writes the target gradient to sm.g; BLOCKS:
-// writes per-block (sum d, sum d^2) to blk_out[G*2]. l_hat and sigma2_hat on every lane.
-template <typename XT, int T, int CPL, int U, bool K, bool GRAD, bool BLOCKS, int MODE = 0,
-          int SPLIT = 1>
-__device__ __forceinline__ bool eval_particle(const WarpEval<XT, T, CPL, U, K> &W, const EstArgs &a,
+// The gradient partials reduced over the row slots of the warp into sm.G1, sm.G2.
+template <int T, int CPL, typename WE, typename CT>
+__device__ __forceinline__ void reduce_partials(const WE &W, CT *g1, CT *g2, WarpSmem<CT> &sm) {
+#pragma unroll
+  for (int s = 0; s < CPL; ++s) {
+#pragma unroll
+    for (int o = T; o < 32; o <<= 1) {
+      g1[s] += __shfl_xor_sync(0xffffffffu, g1[s], o);
+      g2[s] += __shfl_xor_sync(0xffffffffu, g2[s], o);
+    }
+  }
+  if (W.gb == 0) {
+#pragma unroll
+    for (int s = 0; s < CPL; ++s) {
+      sm.G1[W.gl * CPL + s] = g1[s];
+      sm.G2[W.gl * CPL + s] = g2[s];
+    }
+  }
+}
+// The estimates from the sums S of e = d - Ks and Q of e^2 (dbar = S / m), and with GRAD the target
+// gradient into sm.g: delta'(B + C delta / 2) and the gradient column by column.
+template <bool GRAD, typename CT>
+__device__ __forceinline__ void finish_particle(const EstArgs &a, WarpSmem<CT> &sm, double temp,
+                                                double nm, double dbar, double S, double Q, double Ks,
+                                                double &ell, double &sig2) {
+  const int p = a.p, lane = threadIdx.x & 31;
+  double qlin = 0.0;
+  const CT ta = (CT)temp, ta2 = (CT)(temp * temp * nm * nm), tnm = (CT)(temp * nm);
+  const CT cdbar = (CT)dbar;
+  __syncwarp();
+  for (int c = lane; c < p; c += 32) {
+    CT cd = CT(0);
+    for (int k = 0; k < p; ++k) cd = fma(ldg_ct<CT>(a.C_ct, k * p + c), sm.dl[k], cd);
+    const CT bc = ldg_ct<CT>(a.B_ct, c), dc = sm.dl[c];
+    qlin += (double)(dc * (bc + CT(0.5) * cd));
+    if (GRAD)
+      sm.g[c] = target_grad(ta, tnm, ta2, bc, cd, sm.G1[c], sm.G2[c], cdbar,
+                            sm.th[c] - ldg_ct<CT>(a.mu_ct, c), ldg_ct<CT>(a.ivar_ct, c));
+  }
+  qlin = warp_sum(qlin);
+  ell = (a.A_dev ? __ldg(a.A_dev) : a.A) + qlin + nm * fma((double)a.m, Ks, S);
+  sig2 = nm * nm * fmax(0.0, Q - S * S / (double)a.m);
+  __syncwarp();
+}
+
+// One evaluation of the estimator for the warp's particle at theta (in sm.th / sm.dl).
+// Reads rows of idx[0..m); GRAD: writes the target gradient to sm.g; BLOCKS: writes per-block
+// (sum d, sum d^2) to blk_out[G*2]. Returns l_hat and sigma2_hat on every lane.
+template <typename XT, int T, int CPL, int U, bool K, bool GRAD, bool BLOCKS, int MODE = 0>
+__device__ __forceinline__ void eval_particle(const WarpEval<XT, T, CPL, U, K> &W, const EstArgs &a,
                                               const int32_t *idx, WarpSmem<typename Store<XT>::CT> &sm,
                                               double temp, double *blk_out, double &ell,
                                               double &sig2,
-                                              const RowIO<typename Store<XT>::CT> &io_ =
-                                                  RowIO<typename Store<XT>::CT>(),
-                                              int part = 0, int stride = 0) {
+                                              const RowIO<typename Store<XT>::CT> &io =
+                                                  RowIO<typename Store<XT>::CT>()) {
   using CT = typename Store<XT>::CT;
   const XT *Xp = reinterpret_cast<const XT *>(a.Xp);
   const CT inv_s2 = (CT)a.inv_s2;
@@ -437,87 +458,73 @@ __device__ __forceinline__ bool eval_particle(const WarpEval<XT, T, CPL, U, K> &
 #pragma unroll
   for (int s = 0; s < CPL; ++s) g1[s] = g2[s] = CT(0);
   double S, Q, Ks;  // sums of e = d - Ks and e^2, and the shift Ks
-  int j0 = 0, j1 = a.m;
-  RowIO<CT> io = io_;
-  static_assert(SPLIT == 1 || !BLOCKS, "block sums have one order");
-  if constexpr (SPLIT > 1) {
-    split_rows(a.m, part, SPLIT, j0, j1);
-    if (MODE == 1) {
-      io.dsave += j0;
-      io.rsave += j0;
-    }
-  }
-  W.template rows<GRAD, BLOCKS, MODE>(Xp, a.S, a.n, idx + j0, j1 - j0, a.fam, inv_s2, g1, g2,
-                                      blk_out, a.G, S, Q, Ks, a.st, io, a.cv_order == 1);
+  W.template rows<GRAD, BLOCKS, MODE>(Xp, a.S, a.n, idx, a.m, a.fam, inv_s2, g1, g2, blk_out, a.G,
+                                      S, Q, Ks, a.st, io, a.cv_order == 1);
   const double nm = (double)a.n / (double)a.m;
-  if (GRAD) {
-    // reduce the gradient partials over the row slots of the warp
-#pragma unroll
-    for (int s = 0; s < CPL; ++s) {
-#pragma unroll
-      for (int o = T; o < 32; o <<= 1) {
-        g1[s] += __shfl_xor_sync(0xffffffffu, g1[s], o);
-        g2[s] += __shfl_xor_sync(0xffffffffu, g2[s], o);
-      }
-    }
-    if (W.gb == 0) {
-#pragma unroll
-      for (int s = 0; s < CPL; ++s) {
-        sm.G1[W.gl * CPL + s] = g1[s];
-        sm.G2[W.gl * CPL + s] = g2[s];
-      }
-    }
-  }
-  __syncwarp();
-  if constexpr (SPLIT > 1) {
-    // merge: sums about the first warp's shift, S = sum_w (S_w + n_w k_w) and Q = sum_w (Q_w +
-    // k_w (2 S_w + n_w k_w)) with k_w = K_w - K_0 (Chan, Golub & LeVeque 1983), and the gradient
-    // partials' sum e r x likewise
-    __shared__ double merge[8][4];
-    if (W.lane == 0) {
-      merge[part][0] = S;
-      merge[part][1] = Q;
-      merge[part][2] = Ks;
-      merge[part][3] = (double)(j1 - j0);
-    }
-    __syncthreads();
-    if (part) return false;
-    for (int w = 1; w < SPLIT; ++w) {
-      const double nw = merge[w][3], k = nw > 0.0 ? merge[w][2] - Ks : 0.0;
-      S += fma(nw, k, merge[w][0]);
-      Q += merge[w][1] + k * fma(nw, k, 2.0 * merge[w][0]);
-      if (GRAD) {
-        const CT kc = (CT)k;
-        const int off = w * stride / (int)sizeof(CT);
-        for (int c = W.lane; c < a.p; c += 32) {
-          const CT h1 = sm.G1[c + off];
-          sm.G1[c] += h1;
-          sm.G2[c] += fma(kc, h1, sm.G2[c + off]);
-        }
-      }
-    }
-  }
   const double dbar = S / (double)a.m;  // mean of e (the gradient partials hold e r x)
-  // delta'(B + C delta / 2) and, with GRAD, the per-column gradient
-  const int p = a.p;
-  double qlin = 0.0;
-  const CT ta = (CT)temp, ta2 = (CT)(temp * temp * nm * nm), tnm = (CT)(temp * nm);
-  const CT cdbar = (CT)dbar;
-  for (int c = W.lane; c < p; c += 32) {
-    CT cd = CT(0);
-    for (int k = 0; k < p; ++k) cd = fma(ldg_ct<CT>(a.C_ct, k * p + c), sm.dl[k], cd);
-    const CT bc = ldg_ct<CT>(a.B_ct, c), dc = sm.dl[c];
-    qlin += (double)(dc * (bc + CT(0.5) * cd));
+  if (GRAD) reduce_partials<T, CPL>(W, g1, g2, sm);
+  finish_particle<GRAD>(a, sm, temp, nm, dbar, S, Q, Ks, ell, sig2);
+}
+
+// The rows [j0, j1) of a particle that warp w of a CTA takes when the CTA's W warps share one
+// particle: whole sweeps, the parts rounded up, so that the first warp is never without rows (its
+// shift is the merge's).
+__device__ __forceinline__ void split_rows(int m, int w, int W, int &j0, int &j1) {
+  const int n = (m + 31) >> 5;
+  j0 = min(32 * (int)(((int64_t)w * n + W - 1) / W), m);
+  j1 = min(32 * (int)(((int64_t)(w + 1) * n + W - 1) / W), m);
+}
+
+// The same by all WARPS warps of a CTA, for calls with few particles: every warp sums its own rows
+// (split_rows), each with its own sm, `stride` bytes apart, and warp 0 merges them. Returns whether
+// this warp is the one that holds the result.
+template <typename XT, int T, int CPL, int U, int WARPS, bool K, bool GRAD, int MODE = 0>
+__device__ __forceinline__ bool eval_shared(const WarpEval<XT, T, CPL, U, K> &W, const EstArgs &a,
+                                            const int32_t *idx, WarpSmem<typename Store<XT>::CT> &sm,
+                                            double temp, double &ell, double &sig2,
+                                            RowIO<typename Store<XT>::CT> io, int warp, int stride) {
+  using CT = typename Store<XT>::CT;
+  CT g1[CPL], g2[CPL];
+#pragma unroll
+  for (int s = 0; s < CPL; ++s) g1[s] = g2[s] = CT(0);
+  double S, Q, Ks;
+  int j0, j1;
+  split_rows(a.m, warp, WARPS, j0, j1);
+  if (MODE == 1) {
+    io.dsave += j0;
+    io.rsave += j0;
+  }
+  W.template rows<GRAD, false, MODE>(reinterpret_cast<const XT *>(a.Xp), a.S, a.n, idx + j0, j1 - j0,
+                                     a.fam, (CT)a.inv_s2, g1, g2, nullptr, a.G, S, Q, Ks, a.st, io,
+                                     a.cv_order == 1);
+  if (GRAD) reduce_partials<T, CPL>(W, g1, g2, sm);
+  // sums about the first warp's shift, S = sum_w (S_w + n_w k_w) and Q = sum_w (Q_w + k_w (2 S_w +
+  // n_w k_w)) with k_w = K_w - K_0 (Chan, Golub & LeVeque 1983), and the gradient partials' sum e r x
+  // likewise
+  __shared__ double merge[WARPS][4];
+  if (W.lane == 0) {
+    merge[warp][0] = S;
+    merge[warp][1] = Q;
+    merge[warp][2] = Ks;
+    merge[warp][3] = (double)(j1 - j0);
+  }
+  __syncthreads();
+  if (warp) return false;
+  for (int w = 1; w < WARPS; ++w) {
+    const double nw = merge[w][3], k = nw > 0.0 ? merge[w][2] - Ks : 0.0;
+    S += fma(nw, k, merge[w][0]);
+    Q += merge[w][1] + k * fma(nw, k, 2.0 * merge[w][0]);
     if (GRAD) {
-      const CT G1 = sm.G1[c], G2 = sm.G2[c];
-      sm.g[c] = target_grad(ta, tnm, ta2, bc, cd, G1, G2, cdbar, sm.th[c] - ldg_ct<CT>(a.mu_ct, c),
-                            ldg_ct<CT>(a.ivar_ct, c));
+      const CT kc = (CT)k;
+      const int off = w * stride / (int)sizeof(CT);
+      for (int c = W.lane; c < a.p; c += 32) {
+        const CT h1 = sm.G1[c + off];
+        sm.G1[c] += h1;
+        sm.G2[c] += fma(kc, h1, sm.G2[c + off]);
+      }
     }
   }
-  qlin = warp_sum(qlin);
-  ell = (a.A_dev ? __ldg(a.A_dev) : a.A) + qlin + nm * fma((double)a.m, Ks, S);
-  sig2 = nm * nm * fmax(0.0, Q - S * S / (double)a.m);
-  __syncwarp();
+  finish_particle<GRAD>(a, sm, temp, (double)a.n / (double)a.m, S / (double)a.m, S, Q, Ks, ell, sig2);
   return true;
 }
 
@@ -555,60 +562,21 @@ __device__ __forceinline__ int batch_problem(const int *offsets, int nprob, int 
 }
 
 // ------------------------------------------------------------------------------------------------
-// Kernel 1: the plain estimator on caller particles (loglik_est / loglik_grad, cache refresh).
+// Kernel 1: the plain estimator on caller particles (loglik_est / loglik_grad, cache refresh): with the
+// gradient when a.grad is set, with block sums when a.blk is, or both.
 // ------------------------------------------------------------------------------------------------
-// SPLIT = WARPS: one CTA per particle, its warps sharing the rows (few particles); 1: one warp each.
-// GRAD: with the gradient (a.grad); BLOCKS: with the block sums (a.blk). One kernel per use, so that
-// its sweep loop has the instruction cache and the registers to itself (the cache refresh of the
-// 2 x 16-slot tile needs 64 registers instead of 123).
-template <typename XT, int T, int CPL, int U, int WARPS, bool K, int SPLIT, bool GRAD, bool BLOCKS>
-__global__ void __launch_bounds__(WARPS * 32) k_estimate(EstArgs a) {
-  using CT = typename Store<XT>::CT;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5;
-  const int i = SPLIT > 1 ? blockIdx.x : blockIdx.x * WARPS + warp;
-  if (i >= a.B) return;  // whole warp leaves together; without SPLIT no block-level barriers follow
-  WarpEval<XT, T, CPL, U, K> W;
-  const int slots = T * CPL, stride = warp_smem_bytes<XT, T, CPL, U>(a.p);
-  unsigned char *wbase = smem_raw + (size_t)warp * stride;
-  W.init(wbase, a.Yo);
-  WarpSmem<CT> sm(reinterpret_cast<CT *>(wbase + WarpEval<XT, T, CPL, U, K>::RING), a.p, slots);
-  const CT *th = reinterpret_cast<const CT *>(a.theta) + (int64_t)i * a.p;
-  for (int c = W.lane; c < a.p; c += 32) sm.th[c] = th[c];
-  __syncwarp();
-  refresh_delta(W, a, sm);
-  const double temp = a.a_from_state ? a.st->a : a.a_host;
-  const int32_t *idx = a.u + (int64_t)i * a.m;
-  double ell, sig2;
-  double *blk = BLOCKS ? a.blk + (int64_t)i * a.G * 2 : nullptr;
-  if (!eval_particle<XT, T, CPL, U, K, GRAD, BLOCKS, 0, SPLIT>(W, a, idx, sm, temp, blk, ell, sig2,
-                                                               RowIO<CT>(), warp, stride))
-    return;
-  if (GRAD) {
-    CT *g = reinterpret_cast<CT *>(a.grad) + (int64_t)i * a.p;
-    for (int c = W.lane; c < a.p; c += 32) g[c] = sm.g[c];
-  }
-  if (W.lane == 0) {
-    if (a.ell) a.ell[i] = ell;
-    if (a.sig2) a.sig2[i] = sig2;
-    if (!isfinite(ell) || !isfinite(sig2)) set_err(a.st, kErrNonFinite);
-  }
-}
-
-// One warp per particle with all uses in one kernel (chosen by a.grad and a.blk): the gradient of the
-// tiles with eight lanes per row or more, whose schedule alone was slower (p = 101, 16384 particles
-// of m = 5000: 3.53 ms here, 3.87 alone; start of the comparison 3.69).
 template <typename XT, int T, int CPL, int U, int WARPS, bool K>
-__global__ void __launch_bounds__(WARPS * 32) k_estimate_any(EstArgs a) {
+__global__ void __launch_bounds__(WARPS * 32) k_estimate(EstArgs a) {
   using CT = typename Store<XT>::CT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5;
   const int i = blockIdx.x * WARPS + warp;
   if (i >= a.B) return;  // whole warp leaves together; no block-level barriers follow
   WarpEval<XT, T, CPL, U, K> W;
+  const int slots = T * CPL;
   unsigned char *wbase = smem_raw + (size_t)warp * warp_smem_bytes<XT, T, CPL, U>(a.p);
   W.init(wbase, a.Yo);
-  WarpSmem<CT> sm(reinterpret_cast<CT *>(wbase + WarpEval<XT, T, CPL, U, K>::RING), a.p, T * CPL);
+  WarpSmem<CT> sm(reinterpret_cast<CT *>(wbase + WarpEval<XT, T, CPL, U, K>::RING), a.p, slots);
   const CT *th = reinterpret_cast<const CT *>(a.theta) + (int64_t)i * a.p;
   for (int c = W.lane; c < a.p; c += 32) sm.th[c] = th[c];
   __syncwarp();
@@ -637,6 +605,38 @@ __global__ void __launch_bounds__(WARPS * 32) k_estimate_any(EstArgs a) {
   }
 }
 
+// The same for few particles: one CTA per particle, its warps sharing the rows. GRAD: with the
+// gradient (a.grad).
+template <typename XT, int T, int CPL, int U, int WARPS, bool K, bool GRAD>
+__global__ void __launch_bounds__(WARPS * 32) k_estimate_shared(EstArgs a) {
+  using CT = typename Store<XT>::CT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int warp = threadIdx.x >> 5, i = blockIdx.x;
+  WarpEval<XT, T, CPL, U, K> W;
+  const int stride = warp_smem_bytes<XT, T, CPL, U>(a.p);
+  unsigned char *wbase = smem_raw + (size_t)warp * stride;
+  W.init(wbase, a.Yo);
+  WarpSmem<CT> sm(reinterpret_cast<CT *>(wbase + WarpEval<XT, T, CPL, U, K>::RING), a.p, T * CPL);
+  const CT *th = reinterpret_cast<const CT *>(a.theta) + (int64_t)i * a.p;
+  for (int c = W.lane; c < a.p; c += 32) sm.th[c] = th[c];
+  __syncwarp();
+  refresh_delta(W, a, sm);
+  double ell, sig2;
+  if (!eval_shared<XT, T, CPL, U, WARPS, K, GRAD>(W, a, a.u + (int64_t)i * a.m, sm,
+                                                  a.a_from_state ? a.st->a : a.a_host, ell, sig2,
+                                                  RowIO<CT>(), warp, stride))
+    return;
+  if (GRAD) {
+    CT *g = reinterpret_cast<CT *>(a.grad) + (int64_t)i * a.p;
+    for (int c = W.lane; c < a.p; c += 32) g[c] = sm.g[c];
+  }
+  if (W.lane == 0) {
+    if (a.ell) a.ell[i] = ell;
+    if (a.sig2) a.sig2[i] = sig2;
+    if (!isfinite(ell) || !isfinite(sig2)) set_err(a.st, kErrNonFinite);
+  }
+}
+
 // ------------------------------------------------------------------------------------------------
 // Forward/backward pair behind the autograd binding (Sec. 3.2 estimator, its exact gradient for
 // fixed u). Forward: l_hat and sigma2_hat as loglik_est, and per row d_j, r_j saved to
@@ -644,6 +644,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_estimate_any(EstArgs a) {
 //   dL/dtheta = g_l (B + C delta) + sum_j r_j [g_l n/m + g_s 2 (n/m)^2 (d_j - dbar)] x_j
 // from the saved values and the rows gathered again by u (no family terms are re-evaluated).
 // ------------------------------------------------------------------------------------------------
+// SPLIT = WARPS: the CTA's warps share one particle (k_estimate_shared); 1: one warp each.
 template <typename XT, int T, int CPL, int U, int WARPS, bool K, int SPLIT>
 __global__ void __launch_bounds__(WARPS * 32) k_fwdsave(EstArgs a) {
   using CT = typename Store<XT>::CT;
@@ -664,10 +665,14 @@ __global__ void __launch_bounds__(WARPS * 32) k_fwdsave(EstArgs a) {
   io.dsave = reinterpret_cast<CT *>(a.dsave) + (int64_t)i * a.m;
   io.rsave = reinterpret_cast<CT *>(a.rsave) + (int64_t)i * a.m;
   double ell, sig2;
-  if (!eval_particle<XT, T, CPL, U, K, false, false, 1, SPLIT>(W, a, a.u + (int64_t)i * a.m, sm,
-                                                                1.0, nullptr, ell, sig2, io, warp,
-                                                                stride))
-    return;
+  if constexpr (SPLIT > 1) {
+    if (!eval_shared<XT, T, CPL, U, WARPS, K, false, 1>(W, a, a.u + (int64_t)i * a.m, sm, 1.0, ell,
+                                                        sig2, io, warp, stride))
+      return;
+  } else {
+    eval_particle<XT, T, CPL, U, K, false, false, 1>(W, a, a.u + (int64_t)i * a.m, sm, 1.0, nullptr,
+                                                     ell, sig2, io);
+  }
   if (W.lane == 0) {
     a.ell[i] = ell;
     a.sig2[i] = sig2;
@@ -1009,19 +1014,12 @@ inline int launch_tile(int op, const EstArgs &a, cudaStream_t s) {
     if (e == cudaSuccess) kernel<<<grid, block, smem, s>>>(a);
   };
   if (op == 0) {
-    if (a.grad && a.blk) return (int)cudaErrorInvalidValue;  // (no entry point asks for both)
-    if (split) {
-      a.grad ? go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, true, false>)
-             : go(k_estimate<XT, T, CPL, U, WARPS, K, WARPS, false, false>);
-    } else if (a.grad) {
-      if constexpr (T >= 8)
-        go(k_estimate_any<XT, T, CPL, U, WARPS, K>);
-      else
-        go(k_estimate<XT, T, CPL, U, WARPS, K, 1, true, false>);
-    } else {
-      a.blk ? go(k_estimate<XT, T, CPL, U, WARPS, K, 1, false, true>)
-            : go(k_estimate<XT, T, CPL, U, WARPS, K, 1, false, false>);
-    }
+    if (!split)
+      go(k_estimate<XT, T, CPL, U, WARPS, K>);
+    else if (a.grad)
+      go(k_estimate_shared<XT, T, CPL, U, WARPS, K, true>);
+    else
+      go(k_estimate_shared<XT, T, CPL, U, WARPS, K, false>);
   } else if (op == 1) {
     go(k_upm<XT, T, CPL, U, WARPS, K>);
   } else if (op == 2) {
