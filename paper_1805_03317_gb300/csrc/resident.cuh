@@ -647,6 +647,16 @@ inline int launch_res(const EstArgs &a, cudaStream_t s, int sms, bool dry) {
   return (int)cudaGetLastError();
 }
 
+// The groups of a batch run side by side, and an SM takes CTAs of two kernels only if both ask for the
+// same division of its memory. By default that follows from each kernel's own CTAs, so the groups
+// of three small problems ran one after the other or not by a few bytes of a plan: 430 or 485 us
+// per stage (186 particles, p = 5 to 23). All of them ask for the largest shared memory.
+template <typename K> inline void prefer_shared(K *kernel) {
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                           cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+    cudaGetLastError();  // (a hint)
+}
+
 // Batched launch over the problems in b (their largest p, m and G size the plan). dry: check the
 // fit only. Returns a cudaError_t or -2 when the plan does not fit.
 template <typename XT, int CPL, int WARPS>
@@ -661,6 +671,7 @@ inline int launch_res_batch(const BatchArgs &b, int p_max, int m_max, int G_max,
     cudaGetLastError();
     return -2;
   }
+  prefer_shared(k_hmc_res_batch<XT, CPL, WARPS>);
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hmc_res_batch<XT, CPL, WARPS>,
                                                     WARPS * 32, P.total);

@@ -553,6 +553,7 @@ inline int launch_wide_batch(const BatchArgs &b, int p_max, int m_max, int G_max
                              int sms, bool dry) {
   if (p_max > 8 * NV) return -2;
   const WidePlan P = wide_plan<NV>(m_max, G_max);
+  prefer_shared(k_hmc_wide_batch<NV, WARPS>);
   const int per_sm = resident_blocks(k_hmc_wide_batch<NV, WARPS>, (WARPS + 1) * 32, P.total);
   if (per_sm < 1) return -2;
   if (dry || b.total <= 0) return 0;
