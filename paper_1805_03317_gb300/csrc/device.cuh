@@ -277,6 +277,16 @@ __device__ __forceinline__ void horner2<float>(float &pd, float &pr, float D, fl
   pr = v.y;
 }
 
+// a b + c d with a b fused. In FP32 with its roundings written out: left to the compiler, which of the
+// two products is fused depends on the kernel around it, and trajectories of one particle have to
+// come out the same from every kernel.
+__device__ __forceinline__ float two_products(float a, float b, float c, float d) {
+  return __fmaf_rn(a, b, __fmul_rn(c, d));
+}
+__device__ __forceinline__ double two_products(double a, double b, double c, double d) {
+  return c * d + a * b;
+}
+
 // short4: the caller has checked |D| <= 1/20 for every lane of the warp (FP32 only); the
 // logistic series then stops at kappa_6 (truncation below 2e-8 of w|D|^3 and w D^2).
 template <int FAM, typename CT>
@@ -349,9 +359,10 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
       // to its own cancellation (-L1 + sD + wD^2/2) at this |D| in FP32 anyway.
       const float eb = c.c2, eta = eb + D;
       const float e = __expf(-fabsf(eta)), ope = 1.0f + e;
-      const float lb = __logf(fmaxf(sb, 1.0f - sb));
+      const float lb = __log2f(fmaxf(sb, 1.0f - sb));
       const float pos = eb >= 0.0f ? (eta >= 0.0f ? D : -eb) : (eta >= 0.0f ? eta : 0.0f);
-      const float L1f = pos + (__logf(ope) + lb);
+      const float ln2 = 0.693147180559945309f;
+      const float L1f = pos + two_products(lb, ln2, __log2f(ope), ln2);
       const float inv = __fdividef(1.0f, ope);
       const float sg = eta >= 0.0f ? inv : e * inv;
       r = fmaf(w, D, sb - sg);
@@ -379,7 +390,8 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
     // by its series for small |w| (terms w^3 .. w^14: the remainder is below 2e-8 of w^3/3 for
     // |w| <= 1/4 in FP32, below 1e-16 for |w| <= 1/20 in FP64), else directly.
     const CT rb = c.c0, b = c.c1, nu1 = c.c2;
-    const CT w = (D * D - CT(2) * rb * D) * b;
+    const CT w = sizeof(CT) == 4 ? two_products(CT(-2) * rb, D, D, D) * b
+                                 : (D * D - CT(2) * rb * D) * b;
     constexpr CT kSmall = sizeof(CT) == 8 ? CT(0.05) : CT(0.25);
     CT L3;
     if (fabs(w) <= kSmall) {
@@ -401,8 +413,13 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
     r = -c.c0 * fma(CT(0.5) * D, D, t3);
   } else if (FAM == 3) {  // Gaussian, known sd: the expansion is exact; evaluated as written
     const CT res = c.c0;
-    const CT dl = (CT(2) * res * D - D * D) * (CT(0.5) * inv_s2);  // l(eta) - l(eta_bar)
-    d = dl - res * inv_s2 * D + CT(0.5) * inv_s2 * D * D;
+    if constexpr (sizeof(CT) == 4) {  // (l(eta) - l(eta_bar)) - l' D - l'' D^2 / 2
+      const CT h = CT(0.5) * inv_s2;
+      d = two_products(two_products(CT(2) * res, D, -D, D), h, -(res * inv_s2), D) + h * D * D;
+    } else {
+      const CT dl = (CT(2) * res * D - D * D) * (CT(0.5) * inv_s2);  // l(eta) - l(eta_bar)
+      d = dl - res * inv_s2 * D + CT(0.5) * inv_s2 * D * D;
+    }
     r = (res - D) * inv_s2 - res * inv_s2 + inv_s2 * D;
   } else {  // probit: l = log Phi(s*eta)
     const CT s = CT(2) * c.y - CT(1), zb = c.c0, lpb = c.c1, lamb = c.c2, z = zb + s * D;
@@ -410,7 +427,7 @@ __device__ __forceinline__ void row_incr(const RowC<CT> &c, CT D, CT inv_s2, CT 
     log_phi_(z, lp, lam);
     const CT h = lamb * (zb + lamb);  // -l''(eta_bar)
     d = lp - lpb - s * lamb * D + CT(0.5) * h * D * D;
-    r = s * (lam - lamb) + h * D;
+    r = sizeof(CT) == 4 ? two_products(h, D, s, lam - lamb) : s * (lam - lamb) + h * D;
   }
 }
 

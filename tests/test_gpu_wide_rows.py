@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 import torch
 
-from gpu_common import make_pair, state_round, tol
+from gpu_common import device_arrays, make_pair, state_round, tol
 from oracle import oracle as O
 from smc_workloads import small_glm
 
@@ -95,3 +95,43 @@ def test_wide_tiles_cache_after_moves_matches_oracle(family, p, hmc_kernel):
         # absolute per row's d, a block of 52 rows)
         bar = 1e-4 * np.max(np.abs(ref["blocks"][..., k])) + 52 * 3e-7
         assert np.max(np.abs(blk[..., k] - ref["blocks"][..., k])) <= bar
+
+
+def _batch_equals_singles(shapes, kernels, N=40):
+    """A batch of (family, p, m, G) problems, stepped with and without a graph, against the problems
+    alone: particles and cache bit for bit."""
+    wls = [small_glm(f, n=3000, p=p, N=N, m=m, G=G, L=2, x_dtype="bf16", seed=80 + p)
+           for f, p, m, G in shapes]
+    dicts = []
+    for w in wls:
+        X, y = device_arrays(w)
+        dicts.append(dict(X=X, y=y, family=w.family, prior_mean=w.prior_mean,
+                          prior_var=w.prior_var, N=w.N, m=w.m, G=w.G, L=w.L, seed=w.seed,
+                          noise_sigma=w.sigma, dof=w.dof))
+    b = S().smc_batch_init(dicts)
+    got = [S().smc_batch_hmc_kernel(b, q) for q in range(len(wls))]
+    assert got[:len(kernels)] == kernels
+    singles = [make_pair(w, tile_hint=S().smc_batch_tile(b), hmc_kernel=got[q],
+                         theta_bar=S().smc_get_centre(S().smc_batch_context(b, q))[0])[1]
+               for q, w in enumerate(wls)]
+    for use_graph in (False, True):
+        S().smc_batch_stage(b, 1, use_graph=use_graph)
+        for c in singles:
+            S().smc_reweight(c)
+            S().smc_resample(c)
+            S().smc_move(c, 1)
+    for q, c in enumerate(singles):
+        m = S().smc_batch_context(b, q)
+        for x, y in zip((*S().smc_get_particles(m), *S().smc_get_cache(m)),
+                        (*S().smc_get_particles(c), *S().smc_get_cache(c))):
+            assert torch.equal(x, y), q
+        S().smc_free(c)
+    S().smc_batch_free(b)
+
+
+def test_wide_batch_equals_single_problems():
+    """The row terms have one rounding in every kernel (alone and in a batch)."""
+    _batch_equals_singles([("student_t", 50, 700, 20), ("logistic", 56, 300, 7),
+                           ("probit", 41, 200, 5), ("gaussian", 60, 257, 3),
+                           ("student_t", 63, 150, 4), ("poisson", 9, 120, 4)],
+                          [26, 26, 26, 27, 27])
