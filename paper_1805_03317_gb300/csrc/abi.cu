@@ -1898,32 +1898,43 @@ int smc_batch_init(smc_batch **out, int32_t P, const smc_problem *probs, const s
           }
       }
     }
-    std::vector<int> tiles;
-    for (int q = 0; q < P; ++q)
-      if (std::find(tiles.begin(), tiles.end(), gt[q]) == tiles.end()) tiles.push_back(gt[q]);
+    // A group's plan is sized by its largest p, m and G together: a problem that fits alone but not
+    // with the tile's group so far starts another group of that tile.
+    std::vector<std::vector<int>> members;
     b->group_of.assign(P, 0);
+    for (int q = 0; q < P; ++q) {
+      const smc_ctx *c = b->ctx[q];
+      int g = 0;
+      const int ng = (int)b->groups.size();
+      for (; g < ng; ++g) {
+        const BatchGroup &gr = b->groups[g];
+        if (gr.tile != gt[q]) continue;
+        if (gt[q] < 0 || res_launch_batch_bf16(gt[q], dry, std::max(gr.pmax, c->p),
+                                               std::max(gr.mmax, c->m), std::max(gr.Gmax, c->G),
+                                               b->stream, c->sms, true) == 0)
+          break;
+      }
+      if (g == ng) {
+        b->groups.push_back(BatchGroup{gt[q], 0, 0, 0, 0, 0, 0});
+        members.emplace_back();
+      }
+      BatchGroup &gr = b->groups[g];
+      gr.pmax = std::max(gr.pmax, c->p);
+      gr.mmax = std::max(gr.mmax, c->m);
+      gr.Gmax = std::max(gr.Gmax, c->G);
+      members[g].push_back(q);
+      b->group_of[q] = g;
+    }
     std::vector<int> goff(P, 0);
-    for (int t : tiles) {
-      BatchGroup g{t, (int)b->order.size(), 0, 0, 0, 0, 0};
-      for (int q = 0; q < P; ++q) {
-        if (gt[q] != t) continue;
-        const smc_ctx *c = b->ctx[q];
-        b->group_of[q] = (int)b->groups.size();
-        goff[b->order.size()] = g.total;
+    for (size_t g = 0; g < b->groups.size(); ++g) {
+      BatchGroup &gr = b->groups[g];
+      gr.start = (int)b->order.size();
+      for (int q : members[g]) {
+        goff[b->order.size()] = gr.total;
         b->order.push_back(q);
-        g.count += 1;
-        g.total += c->N;
-        g.pmax = std::max(g.pmax, c->p);
-        g.mmax = std::max(g.mmax, c->m);
-        g.Gmax = std::max(g.Gmax, c->G);
+        gr.count += 1;
+        gr.total += b->ctx[q]->N;
       }
-      if (t >= 0 && res_launch_batch_bf16(t, dry, g.pmax, g.mmax, g.Gmax, b->stream,
-                                          b->ctx[0]->sms, true) != 0) {
-        smc_batch_free(b);
-        g_init_error = "batch: a resident group's plan does not fit";
-        return SMC_ERR_ARG;
-      }
-      b->groups.push_back(g);
     }
     if (cudaMalloc(&b->goff_d, sizeof(int) * P) != cudaSuccess ||
         cudaMemcpy(b->goff_d, goff.data(), sizeof(int) * P, cudaMemcpyHostToDevice) != cudaSuccess) {

@@ -135,3 +135,10 @@ def test_wide_batch_equals_single_problems():
                            ("probit", 41, 200, 5), ("gaussian", 60, 257, 3),
                            ("student_t", 63, 150, 4), ("poisson", 9, 120, 4)],
                           [26, 26, 26, 27, 27])
+
+
+def test_batch_group_whose_members_fit_alone_but_not_together():
+    """p = 50 with m = 1500, G = 50 and p = 45 with m = 600, G = 200 each leave room on an SM, a plan
+    of m = 1500 and G = 200 does not: the batch runs them as two groups of one tile."""
+    _batch_equals_singles([("student_t", 50, 1500, 50), ("logistic", 45, 600, 200),
+                           ("student_t", 47, 1490, 40), ("probit", 9, 120, 4)], [26, 26, 26])
