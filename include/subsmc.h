@@ -216,7 +216,10 @@ int smc_stage(smc_ctx *ctx, int32_t R, int32_t use_graph);
 
 /* For B particles: l_hat_m(theta_b; u_b) and sigma2_hat_m(theta_b; u_b).
  * theta: device [B, p] state type; u: device [B, m] int32 row indices in [0, n);
- * ell, sigma2: device [B] double. Out-of-range indices return SMC_ERR_ARG (checked on device). */
+ * ell, sigma2: device [B] double. Out-of-range indices return SMC_ERR_ARG (checked on device).
+ * Rows are summed in one of two orders, chosen by the larger of B and the context's N (up to four
+ * particles per SM, two for FP64 states, or more), so a particle's values do not depend on the rest
+ * of the call as long as B <= N. The same holds for loglik_grad and for loglik_fwd and loglik_bwd. */
 int loglik_est(smc_ctx *ctx, int32_t B, const void *theta, const int32_t *u, double *ell,
                double *sigma2);
 

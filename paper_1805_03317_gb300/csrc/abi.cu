@@ -214,7 +214,16 @@ int hmc_launch(smc_ctx *c, const EstArgs &a) {
   return est_launch_bf16(2, c->tile, a, c->stream);
 }
 
-int est_launch(smc_ctx *c, int op, const EstArgs &a) {
+// The estimator's warps share a particle (eval_shared, estimator.cuh) up to four particles per SM, two
+// for FP64 states; beyond, one warp per particle fills the GPU better than four that repeat the work
+// per particle. us with one warp / shared, gradient: logistic BF16 p = 20, m = 1000: 32 / 23 for 280
+// particles, 32 / 26 for 608, 37 / 42 for 1000; Student-t p = 50, m = 1250: 47 / 31, 49 / 35, 62 / 61;
+// FP64 p = 5, m = 100: 37 / 31, 38 / 47, 62 / 82. The sums differ in their last bits, so what counts
+// is the context's N: a particle's values are the same in every call of up to N particles. (A larger
+// call on a small context takes the line by its own size.)
+int est_launch(smc_ctx *c, int op, const EstArgs &args) {
+  EstArgs a = args;
+  a.few = std::max(a.B, c->N) <= (c->is_f64 ? 2 : 4) * c->sms;
   ProfScope ps(c, op >= 3 ? 0 : op);  // the autograd pair counts as estimator work
   c->launches += 1;
   if (c->x_dtype == SMC_F64) return est_launch_f64(op, c->tile, a, c->stream);

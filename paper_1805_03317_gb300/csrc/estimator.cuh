@@ -993,20 +993,12 @@ __global__ void __launch_bounds__(WARPS * 32) k_hmc_batch(BatchArgs b) {
 // ------------------------------------------------------------------------------------------------
 // Launch helpers
 // ------------------------------------------------------------------------------------------------
-// Particles up to which a CTA's warps share one particle in the estimator kernels: beyond, one warp
-// per particle fills the GPU better than four that repeat the work per particle. us with one warp /
-// shared, gradient: logistic BF16 p = 20, m = 1000: 32 / 23 for 280 particles, 32 / 26 for 608,
-// 37 / 42 for 1000; Student-t p = 50, m = 1250: 47 / 31, 49 / 35, 62 / 61; FP64 p = 5, m = 100:
-// 37 / 31, 38 / 47, 62 / 82.
-template <typename CT> constexpr int kSplitParticles = (sizeof(CT) == 8 ? 2 : 4) * 152;
-
 template <typename XT, int T, int CPL, int U, int WARPS, bool K = false>
 inline int launch_tile(int op, const EstArgs &a, cudaStream_t s) {
   const size_t smem = (size_t)WARPS * warp_smem_bytes<XT, T, CPL, U>(a.p);
   if (a.B <= 0) return 0;
   // (the cache keeps one summation order for every N: the moves start from it)
-  const bool split = WARPS > 1 && (op == 0 || op >= 3) && a.B <= kSplitParticles<typename Store<XT>::CT> &&
-                     !a.blk;
+  const bool split = WARPS > 1 && a.few && (op == 0 || op >= 3) && !a.blk;
   const dim3 grid(split ? a.B : (a.B + WARPS - 1) / WARPS), block(WARPS * 32);
   cudaError_t e = cudaSuccess;
   auto go = [&](auto *kernel) {
