@@ -71,8 +71,7 @@ template <int CPL> __device__ __forceinline__ void load_vec(const double *v, dou
 // Shared-memory plan of one CTA.
 struct ResPlan {
   int rb;    // bytes per resident row (covariates only): an odd multiple of 16 (conflict-free LDS.128)
-  int nvec;  // 16-byte vectors of covariates per row (copied from the packed row)
-  int nvl;   // 16-byte vectors the tile's CPL slots read (>= nvec; the extra ones are zero-filled)
+  int nvl;   // 16-byte vectors the tile's CPL slots read (those past the covariates are zero-filled)
   int off_consts, off_d, off_red, off_redd, off_blk, off_mat, off_k, off_h, total;
 };
 
@@ -81,7 +80,6 @@ struct ResPlan {
 template <typename CT> struct alignas(16) ResK {
   double temp, nm, inv_m;
   CT ta, ta2, tnm;
-  uint32_t smv;
 };
 
 inline __host__ __device__ int round16(int v) { return (v + 15) & ~15; }
@@ -89,8 +87,7 @@ inline __host__ __device__ int round16(int v) { return (v + 15) & ~15; }
 template <typename CT>
 inline ResPlan res_plan(int p, int m, int G, int esz, int warps, int cpl) {
   ResPlan P;
-  const int xb = round16(p * esz), xl = round16(cpl * esz);
-  P.nvec = xb / 16;
+  const int xl = round16(cpl * esz);
   P.nvl = xl / 16;
   P.rb = ((xl / 16) % 2 == 0) ? xl + 16 : xl;
   int off = m * P.rb;
@@ -251,7 +248,6 @@ __device__ __forceinline__ void res_particle(const EstArgs &a, int i, bool reloa
       k.ta = (CT)k.temp;
       k.ta2 = (CT)(k.temp * k.temp * k.nm * k.nm);
       k.tnm = (CT)(k.temp * k.nm);
-      k.smv = smv;
       *ks = k;
     }
     for (int e = tid; e < CPL * CPL; e += NT) {
