@@ -394,7 +394,8 @@ int smc_resample_noalloc(int32_t N, const double *W, uint64_t seed, int32_t stag
  * p, m and G, with one, two or four warps per CTA chosen by p and m (one warp for small
  * subsamples, four for large ones), unless cfgs[q].hmc_kernel = 1 asks for the streamed kernel;
  * problems no resident tile takes (p > 64) and random-walk problems form the streamed group.
- * Problems that share a tile and a warp count share one trajectory launch per move. */
+ * Problems that share a tile and a warp count share one trajectory launch per move, as far as a plan
+ * for the largest p, m and G among them fits; what does not fit opens another launch. */
 typedef struct smc_batch smc_batch;
 int smc_batch_init(smc_batch **out, int32_t P, const smc_problem *probs, const smc_config *cfgs,
                    void *stream);

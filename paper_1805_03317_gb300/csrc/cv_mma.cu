@@ -371,7 +371,7 @@ int launch_fam(const __nv_bfloat16 *Xp, int64_t n, int p, int S, int Yo, double 
   // CTAs per SM by shared memory (1 KB of it per CTA is the system's) and tensor memory. The occupancy
   // query answers 1 for kernels that allocate tensor memory; a tile's phases (copy, FP64 row terms,
   // MMAs, B) follow one another in a CTA, so several CTAs per SM are what overlaps them: logistic
-  // n = 10^6, p = 20: 774 us with one, 393 us with three and one exponential per row.
+  // n = 10^6, p = 20: 774 us with one, 398 us with three and one exponential per row.
   int per_sm = sm_smem / (int)(smem + 1024);
   const int cols = tmem_cols(N);
   if (per_sm * cols > 512) per_sm = 512 / cols;  // every resident CTA gets its columns at once

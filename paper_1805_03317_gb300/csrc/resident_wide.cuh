@@ -19,11 +19,11 @@
 // e = d - K with K the d of the particle's first row. Rows past m are copies of row m - 1 and count
 // as zero. Block sums of the last pass: a block per warp.
 //
-// Bound by latency and issue: eight row warps and the lead at 0.45 instructions per cycle and scheduler
+// Bound by latency and issue: eight row warps and the lead at 0.41 instructions per cycle and scheduler
 // (1250 rows leave room for one CTA per SM), a fifth of the stalls at the three barriers of a pass. us
-// per trajectory of L = 20, streamed and here, Student-t p = 50: 887 and 265 for 280 particles of
-// m = 1250, 550 and 340 for 1024 of 512, 3514 and 3416 for 4096 of 1250, 875 and 820 for 4096 of 100.
-// With four row warps 294, 374, 3780 and 743.
+// per trajectory of L = 20, streamed and here, Student-t p = 50: 770 and 262 for 280 particles of
+// m = 1250, 510 and 340 for 1024 of 512, 3320 and 3350 for 4096 of 1250, 824 and 820 for 4096 of 100
+// (four row warps: 294, 374, 3780 and 743). So every size that fits takes it.
 //
 // Row j is eight 16-byte units; unit u lies at u ^ wide_pos(j), which makes the 128-bit reads of step 1
 // (four lanes x 32 bytes of two rows), the narrow reads of step 2 (32 bytes of four rows, or 16 of
