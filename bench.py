@@ -421,7 +421,7 @@ def full_data_leg(S, wl, dev, R, tc_peak, stages=2, reps=5):
             "tensor_peak_tflops": tc_peak,
             "ms_per_stage": ms_stage,
             "grad_evals_per_s": wl.N * wl.n * R * (wl.L + 1) / (ms_stage / 1e3),
-            "note": "bound by the per-element family terms (3 MUFU ops per particle-row), not the "
+            "note": "bound by the per-element family terms (2 MUFU ops per particle-row), not the "
                     "MMAs"}
 
 
